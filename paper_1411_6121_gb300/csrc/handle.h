@@ -63,7 +63,7 @@ struct dugks_s {
     int cur;               // index of the buffer that holds the current state
     long long *d_step;     // device step counter
     int64_t step;          // host mirror of the step counter
-    double *d_uprev;       // [dim][ncell] velocity at the previous residual
+    double *d_uprev;       // [dim][ncell] velocity at the previous residual (format: launch_residual)
     int have_prev;
     double *d_partials;
     int res_blocks;

@@ -21,11 +21,11 @@
 
 namespace dugks {
 
-// The reduction runs residual_blocks(ncell) blocks, as dugks_residual does: one per 2048
-// cells, at most 4096, each block striding over its cells in a fixed order and writing 8
-// doubles; the final sum takes 8 more. The array holds the 4096 blocks' partials. The entry
+// The reduction runs residual_blocks(ncell) blocks, as dugks_residual does: one per 256
+// cells, at most 608, each block striding over its cells in a fixed order and writing 8
+// doubles; the final sum takes 8 more. The array holds up to 4096 blocks' partials. The entry
 // point accepts meshes up to STATIC_RES_MAX_CELLS = 4096 * 4096 = 16,777,216 cells (a 256^3
-// mesh, at most 4096 cells per block). Size: (4096 + 1) * 8 doubles = 256 KB, held by every
+// mesh). Size: (4096 + 1) * 8 doubles = 256 KB, held by every
 // GPU that loads the library until the process exits.
 constexpr int STATIC_RES_MAX_BLOCKS = 4096;
 constexpr int64_t STATIC_RES_MAX_CELLS = (int64_t)4096 * 4096;
@@ -113,7 +113,7 @@ extern "C" int dugks_residual_static(int32_t lattice, int32_t store, const void 
     p.dt = 2.0;
     p.src = state;
     cudaStream_t st = (cudaStream_t)stream;
-    e = launch_residual(lattice, store, p, 0.0, rt, uprev, have_prev ? 1 : 0, partials, nblocks, final_sum, st);
+    e = launch_residual(lattice, store, p, 0.0, rt, uprev, false, have_prev ? 1 : 0, partials, nblocks, final_sum, st);
     double s[8];
     if (e == cudaSuccess) e = cudaMemcpyAsync(s, final_sum, sizeof s, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
