@@ -294,6 +294,7 @@ int dugks_create(const dugks_mesh *mesh, int32_t lattice, double nu, double dt, 
     ALLOC(h->buf[0], h->state_bytes);
     ALLOC(h->buf[1], h->state_bytes);
     ALLOC(h->d_step, sizeof(long long));
+    if (force->omega != 0.0) { ALLOC(h->d_tfac, sizeof(TimeFactors) * STEP_CHUNK); }
     ALLOC(h->d_uprev, sizeof(double) * dim * h->ncell);
     ALLOC(h->d_partials, sizeof(double) * 8 * h->res_blocks);
     ALLOC(h->d_res, sizeof(double) * 8);
@@ -334,6 +335,7 @@ void dugks_destroy(dugks_t h) {
     cudaFree(h->buf[0]);
     cudaFree(h->buf[1]);
     cudaFree(h->d_step);
+    cudaFree(h->d_tfac);
     cudaFree(h->d_uprev);
     cudaFree(h->d_partials);
     cudaFree(h->d_res);
@@ -380,9 +382,14 @@ static bool clock_on_device(const dugks_t h) {
     return h->force.omega != 0.0 || h->store == DUGKS_STORE_BF16 || h->store == DUGKS_STORE_F16;
 }
 
-// Enqueue n steps starting from the current buffer (no graph).
+// Enqueue n <= STEP_CHUNK steps starting from the current buffer (no graph).
 static int enqueue_steps(dugks_t h, int64_t n) {
     StepParams p = handle_params(h);
+    if (h->d_tfac) {
+        cudaError_t e = launch_time_factors(h->d_step, (int)n, p.omega, p.dt, p.inv_c, h->d_tfac, h->stream);
+        if (e != cudaSuccess) return handle_fail(h, DUGKS_E_CUDA, "time factors: %s", cudaGetErrorString(e));
+        p.tfac = h->d_tfac;
+    }
     int cur = h->cur;
     for (int64_t i = 0; i < n; i++) {
         p.src = h->buf[cur];
@@ -402,7 +409,7 @@ static int enqueue_steps(dugks_t h, int64_t n) {
 int dugks_step(dugks_t h, int64_t n) {
     if (!h || n < 0) return DUGKS_E_INVAL;
     if (n == 0) return DUGKS_OK;
-    const int64_t chunk = 256;  // graph length
+    const int64_t chunk = STEP_CHUNK;  // graph length
     int64_t left = n;
     while (left > 0) {
         const int64_t m = left >= chunk ? chunk : left;
@@ -427,7 +434,7 @@ int dugks_step(dugks_t h, int64_t n) {
             int rc = enqueue_steps(h, m);
             if (rc != DUGKS_OK) return rc;
         }
-        h->launches += m + (clock_on_device(h) ? 1 : 0);
+        h->launches += m + (clock_on_device(h) ? 1 : 0) + (h->d_tfac ? 1 : 0);
         if (m & 1) h->cur ^= 1;
         h->step += m;
         left -= m;

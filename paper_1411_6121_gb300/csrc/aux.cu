@@ -378,6 +378,12 @@ __global__ void __launch_bounds__(32 * RES_SLOTS) residual_final(const double *p
 
 __global__ void advance_kernel(long long *ctr, long long n) { *ctr += n; }
 
+__global__ void time_factors_kernel(const long long *ctr, int n, double omega, double dt, double inv_c,
+                                    TimeFactors *out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = eval_time_factors(omega, dt, inv_c, (double)(*ctr) + (double)i);
+}
+
 static int grid_for(int64_t n, int threads) {
     int64_t b = (n + threads - 1) / threads;
     return (int)(b < 1 ? 1 : (b > 65535 * 8 ? 65535 * 8 : b));
@@ -489,6 +495,12 @@ cudaError_t launch_residual(int q, int store, const StepParams &p, double t, dou
         case 27: return residual_q<27>(store, p, t, rt, uprev, pair, have_prev, partials, nblocks, out, st);
     }
     return cudaErrorNotSupported;
+}
+
+cudaError_t launch_time_factors(const long long *ctr, int n, double omega, double dt, double inv_c, TimeFactors *out,
+                                cudaStream_t st) {
+    time_factors_kernel<<<(n + 31) / 32, 32, 0, st>>>(ctr, n, omega, dt, inv_c, out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_advance(long long *ctr, long long n, cudaStream_t st) {

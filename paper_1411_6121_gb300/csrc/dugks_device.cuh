@@ -257,6 +257,14 @@ __device__ __forceinline__ double rcp_rn(double x) { return __drcp_rn(x); }
 // Parameters of one fused step launch (coefficients precomputed on the host in double;
 // the kernel rounds them once to its arithmetic type).
 // ---------------------------------------------------------------------------------
+// The factors of G(t) and of an oscillating wall pressure at one step: ct = cos(omega t_n) / c
+// (cells), cth = cos(omega (t_n + h)) / c (interfaces) and cwh = cos(omega (t_n + h)), with their
+// FP32 roundings.
+struct TimeFactors {
+    double ct, cth, cwh;
+    float fct, fcth, fcwh;
+};
+
 struct StepParams {
     int nx, ny, nz;
     int64_t px;         // row pitch (elements)
@@ -276,6 +284,7 @@ struct StepParams {
     double omega, dt;          // G(t) = (g + field) cos(omega t)
     const long long *step_ctr; // device step counter: t_n = (*step_ctr + step_off) dt
     int step_off;
+    const TimeFactors *tfac;   // [step_off] the factors of that step, or null: evaluated in the kernel
     int model;                 // 0: incompressible model (eq. (6)); 1: original DUGKS (eq. (5))
     // non-uniform mesh (Sec. 3.4): per axis a, metric[a] = [wf (n+1) | idc (n+1) | idx (n)]:
     // the weight of the high cell at interface i, 1 / (centre distance across i), 1 / (width
@@ -314,12 +323,45 @@ inline void finish_step_params(StepParams &p) {
     for (int i = 0; i < 11; i++) p.fcoef[i] = (float)c[i];
 }
 
+__device__ __forceinline__ TimeFactors eval_time_factors(double omega, double dt, double inv_c, double step) {
+    const double tn = step * dt;
+    TimeFactors f;
+    f.cwh = cos(omega * (tn + 0.5 * dt));
+    f.ct = cos(omega * tn) * inv_c;
+    f.cth = f.cwh * inv_c;
+    f.fct = (float)f.ct;
+    f.fcth = (float)f.cth;
+    f.fcwh = (float)f.cwh;
+    return f;
+}
+
+// Time factors of the step being computed, in the arithmetic type T. Three FP64 cosines per thread
+// took 6 of the 11.5 us of a 128 x 64 step (GB300 runs FP64 at a 64th of its FP32 rate), so
+// sequences of steps read them from a table that one small launch fills (launch_time_factors).
+template <class T>
+__device__ __forceinline__ void time_factors(const StepParams &p, T &ct, T &cth, T &cwh) {
+    if (p.omega == 0.0) {
+        ct = cth = sizeof(T) == 4 ? (T)p.fcoef[2] : (T)p.inv_c;
+        cwh = T(1);
+    } else if (p.tfac) {
+        const TimeFactors *f = p.tfac + p.step_off;
+        if constexpr (sizeof(T) == 4) { ct = __ldg(&f->fct); cth = __ldg(&f->fcth); cwh = __ldg(&f->fcwh); }
+        else { ct = __ldg(&f->ct); cth = __ldg(&f->cth); cwh = __ldg(&f->cwh); }
+    } else {
+        const TimeFactors f = eval_time_factors(p.omega, p.dt, p.inv_c, (double)(*p.step_ctr) + (double)p.step_off);
+        ct = (T)f.ct;
+        cth = (T)f.cth;
+        cwh = (T)f.cwh;
+    }
+}
+
 // Coefficients in the arithmetic type T.
 template <class T>
 struct Coef {
     T rho0, inv_rho0, inv_c, b1, c1, b7, c7, kappa, two_kappa, wcell, wface;
-    T cwh;  // cos(omega (t_n + h)): the time factor of an oscillating wall pressure
-    __device__ __forceinline__ explicit Coef(const StepParams &p) : cwh(T(1)) {
+    T ct, cth;  // cos(omega t_n) / c and cos(omega (t_n + h)) / c: the time factors of G
+    T cwh;      // cos(omega (t_n + h)): the time factor of an oscillating wall pressure
+    __device__ __forceinline__ explicit Coef(const StepParams &p) {
         if constexpr (sizeof(T) == 4) {  // rounded on the host (finish_step_params)
             rho0 = p.fcoef[0]; inv_rho0 = p.fcoef[1]; inv_c = p.fcoef[2]; b1 = p.fcoef[3]; c1 = p.fcoef[4];
             b7 = p.fcoef[5]; c7 = p.fcoef[6]; kappa = p.fcoef[7]; two_kappa = p.fcoef[8]; wcell = p.fcoef[9];
@@ -329,8 +371,7 @@ struct Coef {
             b7 = (T)p.b7; c7 = (T)p.c7; kappa = (T)p.kappa; two_kappa = (T)p.two_kappa; wcell = (T)p.wcell;
             wface = (T)p.wface;
         }
-        if (p.omega != 0.0)
-            cwh = (T)cos(p.omega * (((double)(*p.step_ctr) + (double)p.step_off) * p.dt + 0.5 * p.dt));
+        time_factors<T>(p, ct, cth, cwh);
     }
 };
 

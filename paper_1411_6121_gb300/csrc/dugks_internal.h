@@ -41,6 +41,9 @@ cudaError_t launch_moments(int q, int store, const StepParams &p, double t, doub
 cudaError_t launch_residual(int q, int store, const StepParams &p, double t, double rt, double *uprev, bool pair,
                             int have_prev, double *partials, int nblocks, double *out, cudaStream_t stream);
 int residual_blocks(int64_t ncell);
+// The time factors of the n steps from the device step counter on into out[0 .. n-1].
+cudaError_t launch_time_factors(const long long *ctr, int n, double omega, double dt, double inv_c, TimeFactors *out,
+                                cudaStream_t stream);
 cudaError_t launch_advance(long long *ctr, long long n, cudaStream_t stream);
 
 // Sets the message that dugks_last_error(NULL) returns in this thread (api.cu).

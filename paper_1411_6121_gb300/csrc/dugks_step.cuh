@@ -246,12 +246,7 @@ __device__ __forceinline__ void step_tile(const StepParams &p, int x0, int y0, i
     uint32_t seed = 0;  // stochastic rounding of 16-bit stores
     if constexpr (sizeof(S) == 2) seed = store_seed(*p.step_ctr + p.step_off);
     // time factors of G(t) (reading: cells at t_n, interfaces at t_n + h), over c
-    T ct = (T)p.inv_c, cth = (T)p.inv_c;
-    if (p.omega != 0.0) {
-        const double tn = ((double)(*p.step_ctr) + (double)p.step_off) * p.dt;
-        ct = (T)(cos(p.omega * tn) * p.inv_c);
-        cth = (T)(cos(p.omega * (tn + 0.5 * p.dt)) * p.inv_c);
-    }
+    const T ct = cf.ct, cth = cf.cth;
 
     // Non-uniform mesh metrics (Sec. 3.4): interpolation weight of the high cell at interface i
     // of axis a, 1 / centre distance across it, 1 / width of cell i; hc = h c.

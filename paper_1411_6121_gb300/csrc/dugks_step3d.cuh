@@ -364,12 +364,7 @@ __device__ __forceinline__ void step3d_segment(const StepParams &p, const CUtens
 
     uint32_t seed = 0;  // stochastic rounding of 16-bit stores
     if constexpr (sizeof(S) == 2) seed = store_seed(*p.step_ctr + p.step_off);
-    float ct = p.fcoef[2], cth = p.fcoef[2];
-    if (FORCE && p.omega != 0.0) {
-        const double tn = ((double)(*p.step_ctr) + (double)p.step_off) * p.dt;
-        ct = (float)(cos(p.omega * tn) * p.inv_c);
-        cth = (float)(cos(p.omega * (tn + 0.5 * p.dt)) * p.inv_c);
-    }
+    const float ct = cf.ct, cth = cf.cth;
 
     auto R = [&](int slot, int r, int l) __attribute__((always_inline)) -> float * {
         return ring + ((slot * RY + r) * 32 + l) * CS;

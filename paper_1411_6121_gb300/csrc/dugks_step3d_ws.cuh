@@ -406,12 +406,7 @@ __global__ void __launch_bounds__(512, 1)
     const bool perx = p.bc[0] == 0, pery = p.bc[2] == 0, perz = p.bc[4] == 0;
     const S *src = reinterpret_cast<const S *>(p.src);
     S *dst = reinterpret_cast<S *>(p.dst);
-    float ct = p.fcoef[2], cth = p.fcoef[2];
-    if (FORCE && p.omega != 0.0) {
-        const double tn = ((double)(*p.step_ctr) + (double)p.step_off) * p.dt;
-        ct = (float)(cos(p.omega * tn) * p.inv_c);
-        cth = (float)(cos(p.omega * (tn + 0.5 * p.dt)) * p.inv_c);
-    }
+    const float ct = cf.ct, cth = cf.cth;
     // planes z0 - 1 .. z1 in order: n = pz - (z0 - 1) selects ring slot n % 4 (phase n / 4) and u0
     // slot n % 3
     auto nidx = [&](int pz) __attribute__((always_inline)) { return pz - (z0 - 1); };

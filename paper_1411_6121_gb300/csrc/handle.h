@@ -12,6 +12,8 @@
 
 namespace dugks {
 
+constexpr int STEP_CHUNK = 256;  // most steps of one captured graph
+
 // Checkpoints of a recorded rollout (dugks_record) and the buffers of its adjoint sweep.
 struct AdjointTape {
     int64_t steps = 0;           // recorded steps (0: nothing recorded)
@@ -62,6 +64,7 @@ struct dugks_s {
     void *buf[2];
     int cur;               // index of the buffer that holds the current state
     long long *d_step;     // device step counter
+    dugks::TimeFactors *d_tfac;  // [STEP_CHUNK] time factors of the steps being enqueued (omega != 0)
     int64_t step;          // host mirror of the step counter
     double *d_uprev;       // [dim][ncell] velocity at the previous residual (format: launch_residual)
     int have_prev;
