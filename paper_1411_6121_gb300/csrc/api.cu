@@ -220,8 +220,8 @@ int dugks_create(const dugks_mesh *mesh, int32_t lattice, double nu, double dt, 
             return handle_fail(NULL, DUGKS_E_INVAL, "periodic faces must be paired (axis %d)", d);
         if (lo != DUGKS_BC_PERIODIC && n[d] < 2) return handle_fail(NULL, DUGKS_E_INVAL, "a wall axis needs >= 2 cells");
     }
-    // tile of the reference kernel (tile_x x tile_y cells), or, for the D3Q19 throughput
-    // kernel, tile_y = rows of its 32 x tile_y thread block
+    // tile of the reference kernel (tile_x x tile_y cells), or, for the throughput kernels,
+    // tile_y = rows of their thread block
     const bool thr3d = o.kernel == 0 && (lattice == DUGKS_D3Q19 || lattice == DUGKS_D3Q27) && o.store != DUGKS_STORE_F64;
     const bool thr2d = o.kernel == 0 && lattice == DUGKS_D2Q9 && o.store != DUGKS_STORE_F64;
     int tx = o.tile_x, ty = o.tile_y;
@@ -234,8 +234,8 @@ int dugks_create(const dugks_mesh *mesh, int32_t lattice, double nu, double dt, 
         tx = 32;
         ty = 8;
     } else if (thr2d) {
-        if (ty != 0) ry3d = ty;
-        if (!(ry3d == 4 || ry3d == 8 || ry3d == 16))
+        ry3d = ty;  // 0: chosen by the mesh
+        if (!(ry3d == 0 || ry3d == 4 || ry3d == 8 || ry3d == 16))
             return handle_fail(NULL, DUGKS_E_UNSUPPORTED, "2D kernel rows %d not built", ry3d);
         tx = 32;
         ty = 8;

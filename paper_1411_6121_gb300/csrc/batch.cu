@@ -44,7 +44,7 @@ struct dugks_batch_s {
     long long *d_step = nullptr;
     int64_t step = 0;
     bool timedep = false;
-    bool anyforce = false;  // some instance has an acceleration (uniform or field)
+    int force_mode = 0;     // instances with an acceleration (uniform or field): 0 none, 1 all, 2 some
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int grid = 0;
@@ -99,11 +99,9 @@ cudaError_t launch_batch_s(const dugks_batch_t b, int parity) {
 }
 
 cudaError_t launch_batch(const dugks_batch_t b, int parity) {
-    // throughput tiles: 30 x (ry - 2) inner cells (dugks_step2d.cuh)
-    if (b->tx == 30) {
-        const int ry = b->ty + 2;
-        return launch_step2d_batch(b->d_params, b->d_items, b->nitems, parity, b->store, ry, b->anyforce, b->stream);
-    }
+    // throughput tiles: ty rows (dugks_step2d.cuh)
+    if (b->tx == 30)
+        return launch_step2d_batch(b->d_params, b->d_items, b->nitems, parity, b->store, b->ty + 2, b->force_mode, b->stream);
     switch (b->store) {
         case DUGKS_STORE_F32: return launch_batch_s<float>(b, parity);
         case DUGKS_STORE_BF16: return launch_batch_s<__nv_bfloat16>(b, parity);
@@ -170,10 +168,11 @@ int build_items(dugks_batch_t b) {
         return b->mesh[a].nx * b->mesh[a].ny > b->mesh[c].nx * b->mesh[c].ny;
     });
     std::vector<int4> items;
+    const int cols = b->tx == 30 ? step2d_tile_columns(b->store) : b->tx;
     for (int i : order) {
         const dugks_mesh &m = b->mesh[i];
         for (int64_t y = 0; y < m.ny; y += b->ty)
-            for (int64_t x = 0; x < m.nx; x += b->tx) items.push_back(make_int4(i, (int)x, (int)y, 0));
+            for (int64_t x = 0; x < m.nx; x += cols) items.push_back(make_int4(i, (int)x, (int)y, 0));
     }
     if ((int)items.size() > b->items_cap) {
         cudaFree(b->d_items);
@@ -262,13 +261,15 @@ int dugks_batch_create(int32_t count, const dugks_mesh *meshes, const double *nu
     b->nu.assign(nu, nu + count);
     b->force.assign(forces, forces + count);
     b->bcs.assign(bcs, bcs + count);
+    int forced = 0;
     for (int i = 0; i < count; i++) {
         b->px.push_back((meshes[i].nx + 63) / 64 * 64);  // rows start on 256-byte boundaries
         b->off.push_back(b->elems);
         b->elems += 9 * b->px.back() * meshes[i].ny;
         if (forces[i].omega != 0.0) b->timedep = true;
-        if (forces[i].field || forces[i].g[0] != 0.0 || forces[i].g[1] != 0.0) b->anyforce = true;
+        if (forces[i].field || forces[i].g[0] != 0.0 || forces[i].g[1] != 0.0) forced++;
     }
+    b->force_mode = forced == 0 ? 0 : (forced == count ? 1 : 2);
     // the device clock also seeds the stochastic rounding of 16-bit stores
     if (o.store == DUGKS_STORE_BF16 || o.store == DUGKS_STORE_F16) b->timedep = true;
     b->stream = (cudaStream_t)o.stream;

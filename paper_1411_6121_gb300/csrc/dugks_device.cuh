@@ -227,6 +227,14 @@ __device__ __forceinline__ void store_state_one(S *p0, float v0, uint32_t r) {
     }
 }
 
+// A kernel launched as a programmatic dependent (launch_chained) may start before the work ahead of
+// it in its stream has ended; every thread waits for that work here before it touches memory, and
+// then lets the next such kernel start (which waits in turn).
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
 // Arithmetic type for a storage type: FP32 for FP32/BF16/F16 storage, FP64 for FP64.
 template <class S>
 struct Arith { using T = float; };
@@ -340,7 +348,7 @@ __device__ __forceinline__ TimeFactors eval_time_factors(double omega, double dt
 // sequences of steps read them from a table that one small launch fills (launch_time_factors).
 template <class T>
 __device__ __forceinline__ void time_factors(const StepParams &p, T &ct, T &cth, T &cwh) {
-    if (p.omega == 0.0) {
+    if (__double_as_longlong(p.omega) == 0) {  // (an FP64 comparison would cost more)
         ct = cth = sizeof(T) == 4 ? (T)p.fcoef[2] : (T)p.inv_c;
         cwh = T(1);
     } else if (p.tfac) {

@@ -1,427 +1,820 @@
 // dugks_step2d.cuh -- throughput kernel of the fused DUGKS time step for the D2Q9 velocity
-// set on sm_103a, FP32 arithmetic, F32/BF16/F16 storage.
+// set on sm_103a, FP32 arithmetic, F32 and F16 storage (BF16: dugks_step2d_cell.cuh).
 //
 // Same scheme and readings as the reference kernel in dugks_step.cuh (Appendix steps 1-10
-// of arXiv 1411.6121); the work is organised like the 3D throughput kernel
-// (dugks_step3d.cuh), without its z march:
+// of arXiv 1411.6121). What bounds a 2D step is instruction issue, so the work is arranged to
+// need few instructions per cell:
 //
-//  * A CTA is 32 x RY threads, one per cell (lanes along x, warps along y); the inner
-//    30 x (RY-2) cells are updated, the outer ring is halo. fbar+ (step 1) and its six
-//    moments are made once per cell into shared memory.
-//  * The reconstruction is split per cell, F_k = alpha_k(L) + beta_k(R) with
-//        alpha_k = (1/2 + kappa e_dk) fbar+_k - kappa/4 e_tk C_k,
-//        beta_k  = (1/2 - kappa e_dk) fbar+_k - kappa/4 e_tk C_k
-//    (C_k the central difference of fbar+_k along the tangential axis t), for the six
-//    velocities that cross the interface; the interface moments are the same split taken in
-//    moment space, A(L) + B(R), from the cells' moments and their tangential differences.
-//  * x neighbours exchange beta through warp shuffles, y neighbours through shared memory;
-//    every interface is computed once and both cells use the same bits.
-//  * Wall interfaces take the direct path of dugks_step.cuh (all nine velocities, NEQ,
-//    relax).
-// A launch takes either a grid of tiles (one instance) or a work list of (instance, tile)
-// items walked by a persistent grid (the batched form).
+//  * A block is 32 x RY threads, one warp per row of 64 columns, two neighbouring columns per
+//    lane; the inner 60 x (RY - 2) cells are updated, the rest is halo. The two cells of a lane are
+//    the halves of a float2 and all arithmetic uses the packed FP32 instructions (two FP32
+//    operations each, rounded as the scalar ones). Neighbours along x come by shuffles; along
+//    y each row publishes what its neighbours read in shared memory, behind the only barrier
+//    of a tile without y walls.
+//  * The update of a cell is split into a part linear in fbar+ and the equilibrium (and force)
+//    part of the interface values. With phi = fbar+ and, at an interface, f = (1 - b7) F + W Y
+//    (step 7; F the step-4 value, Y the bracket of b7 f_eq + c7 S), the microflux divergence of
+//    velocity k is (1 - b7) La + W N with
+//      La = sum_d e_d [F(+d) - F(-d)]
+//         = e_x (phi_E - phi_W)/2 - kappa (phi_E - 2 phi + phi_W) + (the same along y)
+//           - kappa/2 e_x e_y [(phi_NE - phi_NW) - (phi_SE - phi_SW)]      (steps 3-4, 8)
+//    formed per velocity from differences of neighbouring cells, and N = sum_d e_d [Y(+d) - Y(-d)].
+//    No step-4 value is formed at an inner interface.
+//  * Y needs the interface moments only (step 6), which are formed in moment space from the cells'
+//    moments: A(L) + B(R) with A, B = M/2 +- kappa M_d - kappa/4 dt M_t. Without a force the
+//    brackets of all six crossing velocities are polynomials of five numbers per interface,
+//      P = base + 4.5 m_n^2/rho0, R = P + 4.5 m_t^2/rho0, S = 9 m_n m_t/rho0, m_n, m_t,
+//    (n the normal, t the tangential axis), so a cell takes the differences of those five
+//    across its two pairs of interfaces and combines them. With a force the six brackets
+//    themselves are differenced. Both cells of an interface use the same numbers, so the
+//    equilibrium flux telescopes exactly.
+//  * At a wall interface step 5 replaces the incoming velocities' F: the interface moments get
+//    the sum of the changes, and the cell's La the changes themselves.
+// Measured (us per step, one instance, before / now; before: one cell per thread, 32 x 8 threads, 30
+// warp instructions per cell, 56% issue): 1024^2 cavity 40.0 / 27.2 (18 instructions per cell, 53%
+// issue, 24 warps per SM), 2048^2 155 / 102, 512 x 256 channel 8.8 / 6.8, 8 x 32 channel 3.45 / 3.4 (the
+// latency of one block).
 #pragma once
 
 #include "dugks_step.cuh"
 
 namespace dugks {
 
-template <int RY, class S = float>
-struct Shape2 {
-    static constexpr int Q = 9;
-    static constexpr int RX = 32;
-    static constexpr int NT = RX * RY;
-    static constexpr int TXI = RX - 2, TYI = RY - 2;  // inner cells
-    static constexpr int NF = n_flux<9>(0);           // crossing velocities per interface (6)
-    static constexpr int NM = 6;                      // moments kept per cell
-    static constexpr int CS = Q + NM;                 // floats per cell (odd: no conflicts)
-    static constexpr int BS = (NF + 3) | 1;           // y exchange: beta_y + B_y
-    static constexpr int FS = NF | 1;                 // y exchange: f at +y
-    static constexpr size_t smem_floats = (size_t)NT * (CS + BS + FS);
-    static constexpr size_t smem_bytes = smem_floats * sizeof(float);
-};
+namespace m2 {
+
+constexpr int TXI = 60;  // columns a tile updates
+// What a row publishes, in float2 per lane: fbar+ of the six velocities with e_y != 0, the x
+// differences of the four diagonals, M_y, M_xy, M_yy, the parts A and B of its y interfaces
+// (drho, j_y, j_x); all linear in fbar+. Then what only the row itself reads: the other
+// fbar+ with e_x != 0 (x walls) and u0 of its update; and, with a force, the acceleration field.
+constexpr int PF = 0, PDX = 6, PM = 10, PA = 13, PB = 16, PX = 19, PU = 21, PFLD = 30;
+template <bool FORCE>
+constexpr int slots() { return FORCE ? PFLD + 2 : PFLD; }
+template <bool FORCE>
+constexpr size_t smem_bytes(int ry) { return sizeof(float2) * 32 * slots<FORCE>() * ry; }
+constexpr int MAX_RY = 16;
+// 80 registers per thread: three blocks of 256 threads (ry 8) or two of 384 (ry 12) per SM
+constexpr int REG_THREADS = 768;
+
+using V = float2;
+__device__ __forceinline__ V bc(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+template <class T>
+__device__ __forceinline__ T all(float x) {
+    if constexpr (sizeof(T) == 4) return x;
+    else return make_float2(x, x);
+}
+__device__ __forceinline__ V add(V a, V b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ V mul(V a, V b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ V fma(V a, V b, V c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ V sub(V a, V b) {
+    V r;
+    asm("{ .reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; sub.rn.f32x2 z, x, y; mov.b64 {%0, %1}, z; }"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+// values of the next and the previous column
+__device__ __forceinline__ V east(V v) { return make_float2(v.y, __shfl_down_sync(0xffffffffu, v.x, 1)); }
+__device__ __forceinline__ V west(V v) { return make_float2(__shfl_up_sync(0xffffffffu, v.y, 1), v.x); }
+// east - west
+__device__ __forceinline__ V cdx(V v) {
+    return make_float2(__fsub_rn(v.y, __shfl_up_sync(0xffffffffu, v.y, 1)),
+                       __fsub_rn(__shfl_down_sync(0xffffffffu, v.x, 1), v.x));
+}
+
+__host__ __device__ constexpr int ex(int k) { return Lat<9>::e(k, 0); }
+__host__ __device__ constexpr int ey(int k) { return Lat<9>::e(k, 1); }
+// position of the diagonal k among 0, 2, 6, 8
+__host__ __device__ constexpr int di(int k) { return k < 3 ? k / 2 : k / 2 - 1; }
+// position of k among the six with e_y != 0 (0, 2, 3, 5, 6, 8)
+__host__ __device__ constexpr int yi(int k) { return k - k / 3 - (k % 3 == 2); }
 
 // Moment slots: 0 M0, 1 M_x, 2 M_y, 3 M_xx, 4 M_yy, 5 M_xy.
-__host__ __device__ constexpr int mslot2_2d(int a, int b) { return a == b ? 3 + a : 5; }
+struct Row {
+    V f[9], m[6], fld[2];  // fbar+, its moments, the cells' acceleration field
+};
 
-// Moments of fbar+ of one cell into m[6], from partial sums over e_a = +1, -1, 0.
-__device__ __forceinline__ void phi_moments_2d(const float f[9], float m[6]) {
-    float sp[2] = {0.0f, 0.0f}, sn[2] = {0.0f, 0.0f}, s0 = 0.0f, mxy = 0.0f;
-    sfor<9>([&](auto kc) {
-        constexpr int k = kc;
-        constexpr int ex = Lat<9>::e(k, 0), ey = Lat<9>::e(k, 1);
-        if constexpr (ex > 0) sp[0] += f[k];
-        if constexpr (ex < 0) sn[0] += f[k];
-        if constexpr (ex == 0) s0 += f[k];
-        if constexpr (ey > 0) sp[1] += f[k];
-        if constexpr (ey < 0) sn[1] += f[k];
-        if constexpr (ex * ey != 0) mxy += ex * ey > 0 ? f[k] : -f[k];
-    });
-    m[0] = s0 + (sp[0] + sn[0]);
-#pragma unroll
-    for (int a = 0; a < 2; a++) {
-        m[1 + a] = sp[a] - sn[a];
-        m[3 + a] = sp[a] + sn[a];
+// What a lane knows of its strip: its first column gx0 (the second is gx0 + 1), the columns it
+// loads (wrapped on a periodic axis, the nearest cell beyond a wall) and where x ghosts lie.
+struct Strip {
+    int lane, gx0, ca, cb;
+    bool vec;       // every lane's two columns load as one aligned pair (the same in all lanes)
+    bool xlo, xhi;  // the strip holds the ghost column below / above an x wall
+};
+
+__device__ __forceinline__ int column(int gx, int nx, bool per) {
+    if (gx >= 0 && gx < nx) return gx;
+    if (per) {
+        const int r = gx % nx;
+        return r < 0 ? r + nx : r;
     }
-    m[5] = mxy;
+    return gx < 0 ? 0 : nx - 1;
 }
 
-// Per-cell parts of the interface normal to d (t = the other axis): alpha, beta for the
-// crossing velocities (compact index), A = (A0, A1x, A1y), B likewise. ph: fbar+ of the cell;
-// m: its moments; C: per-velocity central differences along t (read for the crossing
-// velocities with a component along t); dM: tangential differences of (M_t, M_xt, M_yt).
-template <int d>
-__device__ __forceinline__ void face_parts_2d(const float *ph, const float *m, const float C[9], const float dM[3],
-                                              float kappa, float *alpha, float *beta, float A[3], float B[3]) {
-    constexpr int t = 1 - d;
-    const float qk = -0.25f * kappa;
-    const float g0 = qk * dM[0];
-    A[0] = fmaf(0.5f, m[0], fmaf(kappa, m[1 + d], g0));
-    B[0] = fmaf(0.5f, m[0], fmaf(-kappa, m[1 + d], g0));
+__device__ __forceinline__ Strip make_strip(const StepParams &p, int x0) {
+    Strip s;
+    const bool per = p.bc[0] == 0;
+    s.lane = threadIdx.x & 31;
+    s.gx0 = x0 - 2 + 2 * s.lane;
+    s.ca = column(s.gx0, p.nx, per);
+    s.cb = column(s.gx0 + 1, p.nx, per);
+    s.vec = __all_sync(0xffffffffu, s.cb == s.ca + 1 && (s.ca & 1) == 0);
+    s.xlo = !per && x0 == 0;
+    s.xhi = !per && x0 + TXI >= p.nx;
+    return s;
+}
+
+__device__ __forceinline__ V unpack2(uint32_t w) {  // two F16 values
+    return mul(__half22float2(*reinterpret_cast<const __half2 *>(&w)), bc(F16_UNSCALE));
+}
+
+// The two values as stored, rounded stochastically (store_state_pair): r[15:0] rounds the first,
+// which goes to the low half.
+__device__ __forceinline__ uint32_t f16_pair(V v, uint32_t r) {
+    uint32_t d;
+    asm("cvt.rs.satfinite.f16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.y * F16_SCALE), "f"(v.x * F16_SCALE), "r"(r));
+    return d;
+}
+
+// The lane's stored values of row y (a real row).
+template <class S>
+__device__ __forceinline__ void load_row(const StepParams &p, const Strip &s, int y, V g[9]) {
+    const S *row = reinterpret_cast<const S *>(p.src) + (int64_t)y * p.px;
+    if (s.vec) {
 #pragma unroll
-    for (int a = 0; a < 2; a++) {
-        const float g1 = qk * dM[1 + a];
-        const float mad = m[mslot2_2d(a, d)];
-        A[1 + a] = fmaf(0.5f, m[1 + a], fmaf(kappa, mad, g1));
-        B[1 + a] = fmaf(0.5f, m[1 + a], fmaf(-kappa, mad, g1));
+        for (int k = 0; k < 9; k++) {
+            if constexpr (sizeof(S) == 4) g[k] = __ldg(reinterpret_cast<const float2 *>(row + k * p.dstride + s.ca));
+            else g[k] = unpack2(__ldg(reinterpret_cast<const uint32_t *>(row + k * p.dstride + s.ca)));
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; k++)
+            g[k] = make_float2(Store<S>::ld(row + k * p.dstride + s.ca), Store<S>::ld(row + k * p.dstride + s.cb));
     }
-    sfor<9>([&](auto kc) {
-        constexpr int k = kc;
-        if constexpr (Lat<9>::e(k, d) != 0) {
-            constexpr int i = flux_index<9>(d, k);
-            constexpr int et = Lat<9>::e(k, t);
-            constexpr float ed = (float)Lat<9>::e(k, d);
-            const float f = ph[k];
-            if constexpr (et != 0) {
-                const float gam = qk * (et > 0 ? C[k] : -C[k]);
-                alpha[i] = fmaf(fmaf(kappa, ed, 0.5f), f, gam);
-                beta[i] = fmaf(fmaf(-kappa, ed, 0.5f), f, gam);
-            } else {
-                alpha[i] = mul_rn(fmaf(kappa, ed, 0.5f), f);
-                beta[i] = mul_rn(fmaf(-kappa, ed, 0.5f), f);
-            }
-        }
-    });
 }
 
-// Steps 6-7 for the crossing velocities of the interface normal to d from its step-4 values
-// F (compact) and moments (drho, j): f = F + b7 (geq - F) + c7 S; opposite velocities share
-// e.m and the quadratic part of geq.
-template <int d, bool FORCE>
-__device__ __forceinline__ void face_relax_2d(const Coef<float> &cf, const float *F, float drho, const float j[2],
-                                              const float Gh[2], float *out) {
-    float m[2];
-#pragma unroll
-    for (int a = 0; a < 2; a++) m[a] = FORCE ? fmaf(Gh[a], cf.wface * cf.rho0, j[a]) : j[a];
-    const float m3[3] = {m[0], m[1], 0.0f}, G3[3] = {Gh[0], Gh[1], 0.0f};
-    const float mm = dotD<2, float>(m3, m3);
-    const float base = fmaf(-1.5f * cf.inv_rho0, mm, drho);
-    float gm = 0.0f;
-    if (FORCE) gm = dotD<2, float>(G3, m3) * cf.inv_rho0;
-    const float c45 = 4.5f * cf.inv_rho0;
-    sfor<9>([&](auto kc) {
-        constexpr int k = kc;
-        constexpr int kb = opposite<9>(k);
-        if constexpr (Lat<9>::e(k, d) > 0) {  // the pair (k, kb), e_d = +1 / -1
-            float em = 0.0f, ge = 0.0f;
-#pragma unroll
-            for (int a = 0; a < 2; a++) {
-                if (Lat<9>::e(k, a) > 0) { em += m[a]; if (FORCE) ge += Gh[a]; }
-                if (Lat<9>::e(k, a) < 0) { em -= m[a]; if (FORCE) ge -= Gh[a]; }
-            }
-            constexpr int i = flux_index<9>(d, k), ib = flux_index<9>(d, kb);
-            constexpr float w = Lat<9>::w(k);
-            // interface values need no conservation-exact form (both cells use the same bits)
-            const float q = fmaf(c45 * em, em, base);
-            const float geq = mul_rn(w, fmaf(em, 3.0f, q)), geqb = mul_rn(w, fmaf(em, -3.0f, q));
-            float v = fmaf(cf.b7, geq - F[i], F[i]), vb = fmaf(cf.b7, geqb - F[ib], F[ib]);
-            if (FORCE) {
-                v = fmaf(cf.c7 * 3.0f * (ge - gm), fmaf(w, cf.rho0, geq), v);
-                vb = fmaf(cf.c7 * 3.0f * (-ge - gm), fmaf(w, cf.rho0, geqb), vb);
-            }
-            out[i] = v;
-            out[ib] = vb;
-        }
-    });
+// The ghost columns beyond x walls (step 2, reading R3: 2 f0 - f1).
+__device__ __forceinline__ V x_ghost(V v, const Strip &s, int nx) {
+    if (s.xlo) {
+        const float a = __shfl_down_sync(0xffffffffu, v.x, 1), b = __shfl_down_sync(0xffffffffu, v.y, 1);
+        if (s.gx0 == -2) v.y = ghost_value(a, b);
+    }
+    if (s.xhi) {
+        const float a = __shfl_up_sync(0xffffffffu, v.y, 1), b = __shfl_up_sync(0xffffffffu, v.x, 1);
+        if (s.gx0 == nx) v.x = ghost_value(a, b);
+        if (s.gx0 == nx - 1) v.y = ghost_value(v.x, a);
+    }
+    return v;
 }
 
-// One tile: inner cells [x0, x0 + 30) x [y0, y0 + RY - 2) of the instance p.
-template <class S, int RY, bool FORCE>
-__device__ __forceinline__ void step2d_tile(const StepParams &p, unsigned char *smem_raw, int x0, int y0) {
-    using K = Shape2<RY, S>;
-    constexpr int Q = 9, NF = K::NF, CS = K::CS;
-    float *cell = reinterpret_cast<float *>(smem_raw);  // [RY][32][CS]: fbar+ then moments
-    float *xb = cell + K::NT * CS;                      // [RY][32][BS]: beta_y, B_y
-    float *xf = xb + K::NT * K::BS;                     // [RY][32][FS]: f at +y
-    const Coef<float> cf(p);
-
-    const int lane = threadIdx.x, row = threadIdx.y;
-    const int nx = p.nx, ny = p.ny;
-    const int gx = x0 - 1 + lane, gy = y0 - 1 + row;
-    const int64_t ncell = (int64_t)nx * ny;
-    const bool perx = p.bc[0] == 0, pery = p.bc[2] == 0;
-    const S *src = reinterpret_cast<const S *>(p.src);
-    S *dst = reinterpret_cast<S *>(p.dst);
-
-    // cell classification (as in the 3D kernel)
-    const bool inner = lane >= 1 && lane <= K::TXI && row >= 1 && row <= K::TYI;
-    const bool upd = inner && gx < nx && gy < ny;
-    int cx = gx, cy = gy;
-    bool load = true;
-    if (gx < 0 || gx >= nx) { if (perx && gx >= -1 && gx <= nx) cx = wrap_idx(gx, nx); else load = false; }
-    if (gy < 0 || gy >= ny) { if (pery && gy >= -1 && gy <= ny) cy = wrap_idx(gy, ny); else load = false; }
-    const bool yreal = (gy >= 0 && gy < ny) || (pery && gy >= -1 && gy <= ny);
-    const bool xghost = !perx && (gx == -1 || gx == nx) && yreal;
-    const bool yghost = !pery && (gy == -1 || gy == ny) && gx >= -1 && gx <= nx;
-    const bool xwall_tile = !perx && (x0 == 0 || x0 + K::TXI >= nx);
-    const bool ywall_tile = !pery && (y0 == 0 || y0 + K::TYI >= ny);
-    const bool need_x = row >= 1 && row <= K::TYI && gy >= 0 && gy < ny && lane <= K::TXI && gx >= -1 && gx < nx;
-    const bool ycol = lane >= 1 && lane <= K::TXI && gx >= 0 && gx < nx && gy >= -1 && gy <= ny;
-    const bool need_y = ycol && row <= K::TYI && gy < ny;
-
-    uint32_t seed = 0;  // stochastic rounding of 16-bit stores
-    if constexpr (sizeof(S) == 2) seed = store_seed(*p.step_ctr + p.step_off);
-    const float ct = cf.ct, cth = cf.cth;
-    auto Rp = [&](int r, int l) __attribute__((always_inline)) -> float * { return cell + (r * 32 + l) * CS; };
-
-    // interface acceleration / c at t+h between (x, y) - e_d and (x, y) (reading R2)
-    auto faceG = [&](int d, int x, int y, float Gh[2]) __attribute__((always_inline)) {
-        int lo[2] = {x, y}, hi[2] = {x, y};
-        const int nd = d == 0 ? nx : ny;
-        const bool per = d == 0 ? perx : pery;
-        lo[d] -= 1;
-        if (per) { lo[d] = wrap_idx(lo[d], nd); hi[d] = wrap_idx(hi[d], nd); }
-        else { lo[d] = max(lo[d], 0); hi[d] = min(hi[d], nd - 1); }
-        const int64_t il = (int64_t)lo[0] + (int64_t)nx * lo[1], ih = (int64_t)hi[0] + (int64_t)nx * hi[1];
+// Row y (a real row) from its stored values g: step 1 (eq. (24)) with the rounding of
+// moments<9, float, true> and relax, the moments of fbar+, and x ghosts. With d = fbar+ - g~,
+// u0 = g~ + 4/3 d (eq. (25): 4/3 fbar+ - 1/3 g~).
+template <bool FORCE>
+__device__ __forceinline__ void make_row(const StepParams &p, const Coef<float> &cf, const Strip &s, int y,
+                                         const V g[9], Row &r, V u0[9]) {
+    V G[2] = {bc(0.0f), bc(0.0f)};
+    r.fld[0] = r.fld[1] = bc(0.0f);
+    if constexpr (FORCE) {
+        if (p.field) {
+            const float *fr = p.field + (int64_t)p.nx * y;
+            const int64_t ncell = (int64_t)p.nx * p.ny;
 #pragma unroll
-        for (int a = 0; a < 2; a++) {
-            float v = p.fg[a];
-            if (p.field) v += 0.5f * (__ldg(p.field + a * ncell + il) + __ldg(p.field + a * ncell + ih));
-            Gh[a] = v * cth;
+            for (int a = 0; a < 2; a++) r.fld[a] = make_float2(__ldg(fr + a * ncell + s.ca), __ldg(fr + a * ncell + s.cb));
         }
-    };
-
-    // ---- step 1 for the own cell; g and fbar+ stay in registers for the update ----
-    float g[Q], f[Q];
+#pragma unroll
+        for (int a = 0; a < 2; a++) G[a] = mul(add(bc(p.fg[a]), r.fld[a]), bc(cf.ct));
+    }
+    V drho = g[0];
+#pragma unroll
+    for (int k = 1; k < 9; k++) drho = add(drho, g[k]);
+    float ax = 0.0f, ay = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        if (k == 4) continue;
+        ax = fmaxf(ax, fabsf(g[k].x));
+        ay = fmaxf(ay, fabsf(g[k].y));
+    }
+    const V sp = make_float2(__uint_as_float((__float_as_uint(ax) & 0x7f800000u) + 0x02c00000u),
+                             __uint_as_float((__float_as_uint(ay) & 0x7f800000u) + 0x02c00000u));
+    V hi[2] = {bc(0.0f), bc(0.0f)}, lo[2] = {bc(0.0f), bc(0.0f)};
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        if (k == 4) continue;
+        const V h = sub(add(g[k], sp), sp), l = sub(g[k], h);
+        if (ex(k) > 0) { hi[0] = add(hi[0], h); lo[0] = add(lo[0], l); }
+        if (ex(k) < 0) { hi[0] = sub(hi[0], h); lo[0] = sub(lo[0], l); }
+        if (ey(k) > 0) { hi[1] = add(hi[1], h); lo[1] = add(lo[1], l); }
+        if (ey(k) < 0) { hi[1] = sub(hi[1], h); lo[1] = sub(lo[1], l); }
+    }
+    V m[2];
+#pragma unroll
+    for (int a = 0; a < 2; a++) m[a] = add(hi[a], FORCE ? fma(G[a], bc(cf.wcell * cf.rho0), lo[a]) : lo[a]);
+    const V mm = fma(m[0], m[0], mul(m[1], m[1]));
+    V gm = bc(0.0f);
+    if constexpr (FORCE) gm = mul(fma(G[0], m[0], mul(G[1], m[1])), bc(cf.inv_rho0));
+    const V base = fma(bc(-1.5f * cf.inv_rho0), mm, drho), c45 = bc(4.5f * cf.inv_rho0);
+    const V b1 = bc(cf.b1), b43 = bc(cf.b1 * (4.0f / 3.0f)), t43 = bc(4.0f / 3.0f);
+    sfor<4>([&](auto jc) {
+        constexpr int k = 5 + jc;  // (0, 1), (1, -1), (1, 0), (1, 1) and the opposite of each
+        constexpr double W = Lat<9>::wt<double>(k);
+        constexpr float wh = (float)W, wl = (float)(W - (double)wh);
+        constexpr float w3h = (float)(3.0 * W), w3l = (float)(3.0 * W - (double)w3h);
+        const V em = ex(k) == 0 ? m[1] : (ey(k) == 0 ? m[0] : (ey(k) > 0 ? add(m[0], m[1]) : sub(m[0], m[1])));
+        const V q = fma(mul(c45, em), em, base);
+        const V wq = fma(bc(wl), q, mul(bc(wh), q));
+        const V en = sub(bc(0.0f), em);
+        const V gp = fma(bc(w3h), em, fma(bc(w3l), em, wq)), gn = fma(bc(w3h), en, fma(bc(w3l), en, wq));
+        const V dp = sub(gp, g[k]), dn = sub(gn, g[8 - k]);
+        if constexpr (!FORCE) {
+            r.f[k] = fma(b1, dp, g[k]);
+            r.f[8 - k] = fma(b1, dn, g[8 - k]);
+            u0[k] = fma(b43, dp, g[k]);
+            u0[8 - k] = fma(b43, dn, g[8 - k]);
+        } else {
+            const V ge = ex(k) == 0 ? G[1] : (ey(k) == 0 ? G[0] : (ey(k) > 0 ? add(G[0], G[1]) : sub(G[0], G[1])));
+            const V fqp = fma(bc((float)W), bc(cf.rho0), gp), fqn = fma(bc((float)W), bc(cf.rho0), gn);
+            const V c3 = bc(3.0f * cf.c1), n3 = bc(-3.0f * cf.c1);
+            const V ip = fma(mul(c3, sub(ge, gm)), fqp, mul(b1, dp)), in = fma(mul(n3, add(ge, gm)), fqn, mul(b1, dn));
+            r.f[k] = add(g[k], ip);
+            r.f[8 - k] = add(g[8 - k], in);
+            u0[k] = fma(t43, ip, g[k]);
+            u0[8 - k] = fma(t43, in, g[8 - k]);
+        }
+    });
     {
-        float *o = Rp(row, lane);
-        if (load) {
-            const int64_t off = (int64_t)cy * p.px + cx;
-#pragma unroll
-            for (int k = 0; k < Q; k++) g[k] = (float)Store<S>::ld(src + k * p.dstride + off);
-            float Gh[3] = {0.0f, 0.0f, 0.0f}, drho, m[3];
-            if (FORCE) cell_G<2, float>(p, (int64_t)cx + (int64_t)nx * cy, ncell, ct, Gh);
-            moments<Q, float, true>(g, Gh, cf.wcell * cf.rho0, drho, m);
-            relax<Q, float, FORCE>(g, drho, m, Gh, cf.rho0, cf.inv_rho0, cf.b1, cf.c1, f);
-            float mo[6];
-            phi_moments_2d(f, mo);
-#pragma unroll
-            for (int k = 0; k < Q; k++) o[k] = f[k];
-#pragma unroll
-            for (int i = 0; i < 6; i++) o[Q + i] = mo[i];
-        } else {
-#pragma unroll
-            for (int k = 0; k < CS; k++) o[k] = 0.0f;
-#pragma unroll
-            for (int k = 0; k < Q; k++) g[k] = f[k] = 0.0f;
-        }
+        constexpr double W = Lat<9>::wt<double>(4);
+        constexpr float wh = (float)W, wl = (float)(W - (double)wh);
+        const V gq = fma(bc(wl), base, mul(bc(wh), base));
+        V in = mul(b1, sub(gq, g[4]));
+        if constexpr (FORCE) in = fma(mul(bc(-3.0f * cf.c1), gm), fma(bc((float)W), bc(cf.rho0), gq), in);
+        r.f[4] = add(g[4], in);
+        u0[4] = fma(t43, in, g[4]);
     }
-    // step 2 (reading R3: ghost = 2 f0 - f1, x then y): fbar+ and its moments
-    if (xwall_tile) {
-        __syncthreads();
-        if (xghost) {
-            const int d1 = gx < 0 ? 1 : -1;
-            float *o = Rp(row, lane);
-            const float *a = Rp(row, lane + d1), *b = Rp(row, lane + 2 * d1);
+    const V xp = add(add(r.f[6], r.f[7]), r.f[8]), xn = add(add(r.f[0], r.f[1]), r.f[2]);
+    const V yp = add(add(r.f[2], r.f[5]), r.f[8]), yn = add(add(r.f[0], r.f[3]), r.f[6]);
+    r.m[0] = add(add(add(r.f[3], r.f[4]), r.f[5]), add(xp, xn));
+    r.m[1] = sub(xp, xn);
+    r.m[2] = sub(yp, yn);
+    r.m[3] = add(xp, xn);
+    r.m[4] = add(yp, yn);
+    r.m[5] = add(sub(sub(r.f[0], r.f[2]), r.f[6]), r.f[8]);
+    if (s.xlo || s.xhi) {  // warp-uniform; only the columns' values that x neighbours read
 #pragma unroll
-            for (int k = 0; k < CS; k++) o[k] = ghost_value(a[k], b[k]);
-        }
-    }
-    if (ywall_tile) {
-        __syncthreads();
-        if (yghost) {
-            const int d1 = gy < 0 ? 1 : -1;
-            float *o = Rp(row, lane);
-            const float *a = Rp(row + d1, lane), *b = Rp(row + 2 * d1, lane);
+        for (int k = 0; k < 9; k++)
+            if (ex(k) != 0) r.f[k] = x_ghost(r.f[k], s, p.nx);
 #pragma unroll
-            for (int k = 0; k < CS; k++) o[k] = ghost_value(a[k], b[k]);
-        }
+        for (int i = 0; i < 6; i++) r.m[i] = x_ghost(r.m[i], s, p.nx);
     }
-    __syncthreads();
+}
 
-    // direct path for one interface (walls): all velocities from shared memory, NEQ, relax.
-    // Interface normal to d between the own cell and its +d neighbour; gfd its index along d.
-    auto direct_face = [&](int d, int gfd, float *out) {
-        auto rec = [&](int r, int l, float F[Q]) __attribute__((always_inline)) {
-            // interface normal to d whose low cell is (r, l)
-            if (d == 0)
-                reconstruct<Q, 0, float>(Rp(r, l), Rp(r, l + 1), Rp(r - 1, l), Rp(r - 1, l + 1), Rp(r + 1, l),
-                                         Rp(r + 1, l + 1), Rp(r, l), Rp(r, l + 1), Rp(r, l), Rp(r, l + 1), cf.kappa, F);
-            else
-                reconstruct<Q, 1, float>(Rp(r, l), Rp(r + 1, l), Rp(r, l - 1), Rp(r + 1, l - 1), Rp(r, l + 1),
-                                         Rp(r + 1, l + 1), Rp(r, l), Rp(r + 1, l), Rp(r, l), Rp(r + 1, l), cf.kappa, F);
+// Per-cell parts of the moments at the interface normal to n (mn, mt: slots of M_n, M_t; mnn,
+// mnt: of M_nn, M_nt), in the order drho, j_n, j_t; D: differences along t of (M_t, M_nt, M_tt).
+template <int SIGN>
+__device__ __forceinline__ void moment_parts(float kappa, V m0, V mn, V mt, V mnn, V mnt, const V D[3], V out[3]) {
+    const V h = bc(0.5f), k = bc(SIGN > 0 ? kappa : -kappa), q = bc(-0.25f * kappa);
+    out[0] = fma(h, m0, fma(k, mn, mul(q, D[0])));
+    out[1] = fma(h, mn, fma(k, mnn, mul(q, D[1])));
+    out[2] = fma(h, mt, fma(k, mnt, mul(q, D[2])));
+}
+__device__ __forceinline__ void x_diffs(const V m[6], V D[3]) {  // of (M_x, M_xy, M_xx)
+    D[0] = cdx(m[1]);
+    D[1] = cdx(m[5]);
+    D[2] = cdx(m[3]);
+}
+
+// The numbers of an interface that its two cells difference (header): without a force P, R, S,
+// m_n, m_t; with one the brackets Y of the six crossing velocities (n, t) = (1, 0), (-1, 0),
+// (1, 1), (-1, -1), (1, -1), (-1, 1). fm: drho, j_n, j_t; Gn, Gt: the acceleration / c there.
+template <bool FORCE>
+__device__ __forceinline__ void face_numbers(const Coef<float> &cf, const V fm[3], V Gn, V Gt, V out[6]) {
+    const float c45 = 4.5f * cf.inv_rho0;
+    V mn = fm[1], mt = fm[2];
+    if constexpr (FORCE) {
+        const V w = bc(cf.wface * cf.rho0);
+        mn = fma(Gn, w, mn);
+        mt = fma(Gt, w, mt);
+    }
+    const V base = fma(bc(-1.5f * cf.inv_rho0), fma(mn, mn, mul(mt, mt)), fm[0]);
+    const V P = fma(mul(bc(c45), mn), mn, base);
+    const V R = fma(mul(bc(c45), mt), mt, P);
+    const V S = mul(mul(bc(2.0f * c45), mn), mt);
+    if constexpr (!FORCE) {
+        out[0] = P;
+        out[1] = R;
+        out[2] = S;
+        out[3] = mn;
+        out[4] = mt;
+    } else {
+        // Y = b7 X + t (rho0 + X), X = f_eq / W - rho0 the velocity's even part q +- 3 e.m,
+        // t = 3 c7 (G.e - G.m/rho0)
+        const V c73 = bc(3.0f * cf.c7), b7 = bc(cf.b7), r0 = bc(cf.rho0);
+        const V gm = mul(c73, mul(fma(Gn, mn, mul(Gt, mt)), bc(cf.inv_rho0)));
+        auto pair = [&](V q, V em, V ge, V &yp, V &yn) __attribute__((always_inline)) {
+            const V e3 = mul(bc(3.0f), em), g3 = mul(c73, ge);
+            const V Xp = add(q, e3), Xn = sub(q, e3);
+            const V tp = sub(g3, gm), tn = mul(bc(-1.0f), add(g3, gm));
+            yp = fma(tp, add(r0, Xp), mul(b7, Xp));
+            yn = fma(tn, add(r0, Xn), mul(b7, Xn));
         };
-        float F[Q];
-        rec(row, lane, F);
-        const int nd = d == 0 ? nx : ny;
-        const bool per = d == 0 ? perx : pery;
-        const int wall = !per && (gfd == 0 || gfd == nd);
-        float Gb[3] = {0.0f, 0.0f, 0.0f}, Gc[3] = {0.0f, 0.0f, 0.0f};
-        const int fx = d == 0 ? gfd : min(max(gx, 0), nx - 1);
-        const int fy = d == 1 ? gfd : min(max(gy, 0), ny - 1);
-        if (FORCE) faceG(d, fx, fy, Gb);
-        float Fc[Q];
-        if (wall) {
-            // x_c: the boundary cell's opposite interface, one cell inward (reading R4)
-            const int sh = gfd == 0 ? 1 : -1;
-            if (d == 0) rec(row, lane + sh, Fc);
-            else rec(row + sh, lane, Fc);
-            if (FORCE) faceG(d, d == 0 ? gfd + sh : fx, d == 1 ? gfd + sh : fy, Gc);
-        }
-        if (d == 0) interface_f<Q, 0, float, false>(p, cf, F, Gb, wall, gfd == 0 ? 0 : 1, Fc, Gc, out);
-        else interface_f<Q, 1, float, false>(p, cf, F, Gb, wall, gfd == 0 ? 0 : 1, Fc, Gc, out);
-    };
-
-    // central differences along t of the own cell: per velocity (diagonals only) and of
-    // the moments (M_t, M_xt, M_yt)
-    auto cdiff = [&](auto tc, float C[Q], float dM[3]) __attribute__((always_inline)) {
-        constexpr int t = decltype(tc)::value;
-        const float *lo, *hi;
-        if constexpr (t == 0) { lo = Rp(row, max(lane - 1, 0)); hi = Rp(row, min(lane + 1, 31)); }
-        else { lo = Rp(max(row - 1, 0), lane); hi = Rp(min(row + 1, RY - 1), lane); }
-        sfor<Q>([&](auto kc) {
-            constexpr int k = kc;
-            if constexpr (Lat<9>::e(k, 0) != 0 && Lat<9>::e(k, 1) != 0) C[k] = hi[k] - lo[k];
-            else C[k] = 0.0f;
-        });
-        dM[0] = hi[Q + 1 + t] - lo[Q + 1 + t];
-#pragma unroll
-        for (int a = 0; a < 2; a++) dM[1 + a] = hi[Q + mslot2_2d(a, t)] - lo[Q + mslot2_2d(a, t)];
-    };
-    constexpr std::integral_constant<int, 0> AX{};
-    constexpr std::integral_constant<int, 1> AY{};
-    const float *cur = Rp(row, lane);
-
-    // ---- x interfaces (beta parts exchanged by shuffles) ----
-    float fxp[NF];
-#pragma unroll
-    for (int i = 0; i < NF; i++) fxp[i] = 0.0f;
-    if (row >= 1 && row <= K::TYI) {  // warp-uniform: halo rows own no x interface
-        float alx[NF], bex[NF], Ax[3], Bx[3], Cy[Q], dy[3];
-        cdiff(AY, Cy, dy);
-        face_parts_2d<0>(cur, cur + Q, Cy, dy, cf.kappa, alx, bex, Ax, Bx);
-        float F[NF], jb[2];
-#pragma unroll
-        for (int i = 0; i < NF; i++) F[i] = alx[i] + __shfl_down_sync(0xffffffffu, bex[i], 1);
-        const float drb = Ax[0] + __shfl_down_sync(0xffffffffu, Bx[0], 1);
-#pragma unroll
-        for (int a = 0; a < 2; a++) jb[a] = Ax[1 + a] + __shfl_down_sync(0xffffffffu, Bx[1 + a], 1);
-        if (need_x) {
-            if (!perx && (gx == -1 || gx == nx - 1)) {
-                float t[NF];
-                direct_face(0, gx + 1, t);
-#pragma unroll
-                for (int i = 0; i < NF; i++) fxp[i] = t[i];
-            } else {
-                float Gb[2] = {0.0f, 0.0f};
-                if (FORCE) {
-                    float G3[3];
-                    faceG(0, gx + 1, gy, G3);
-                    Gb[0] = G3[0];
-                    Gb[1] = G3[1];
-                }
-                face_relax_2d<0, FORCE>(cf, F, drb, jb, Gb, fxp);
-            }
-        }
+        pair(P, mn, Gn, out[0], out[1]);
+        pair(add(R, S), add(mn, mt), add(Gn, Gt), out[2], out[3]);
+        pair(sub(R, S), sub(mn, mt), sub(Gn, Gt), out[4], out[5]);
     }
-    // ---- y interfaces: publish beta_y, B_y; then the interface above the own cell ----
-    float aly[NF], Ay[3];
-    if (ycol) {
-        float bey[NF], By[3], Cx[Q], dx[3];
-        cdiff(AX, Cx, dx);
-        face_parts_2d<1>(cur, cur + Q, Cx, dx, cf.kappa, aly, bey, Ay, By);
-        float *b = xb + (row * 32 + lane) * K::BS;
-#pragma unroll
-        for (int i = 0; i < NF; i++) b[i] = bey[i];
-#pragma unroll
-        for (int i = 0; i < 3; i++) b[NF + i] = By[i];
+}
+
+// f_eq deviation of velocity k over the cells (geq_k).
+template <int k, class T>
+__device__ __forceinline__ T geq2(const Coef<float> &cf, T dr, T mx, T my) {
+    const float ir = cf.inv_rho0;
+    const T mm = fma(mx, mx, mul(my, my));
+    T em = all<T>(0.0f);
+    if (ex(k) > 0) em = mx;
+    if (ex(k) < 0) em = mul(all<T>(-1.0f), mx);
+    if (ey(k) > 0) em = ex(k) ? add(em, my) : my;
+    if (ey(k) < 0) em = ex(k) ? sub(em, my) : mul(all<T>(-1.0f), my);
+    const T x = fma(em, all<T>(3.0f), fma(mul(all<T>(ir), em), mul(all<T>(4.5f), em), fma(all<T>(-1.5f * ir), mm, dr)));
+    constexpr double W = Lat<9>::wt<double>(k);
+    constexpr float wh = (float)W, wl = (float)(W - (double)wh);
+    return fma(all<T>(wl), x, mul(all<T>(wh), x));
+}
+
+// Step 5 for the incoming velocities kin[0..2] (t component -1, 0, 1) of a wall normal to axis d:
+// their new values minus the step-4 ones. Fi, Fo: step-4 values of the incoming velocities and of
+// their opposites at the wall; Fc at x_c; cm: drho, j_n, j_t at x_c; Gc: acceleration / c there.
+// Adds the change to the wall's moments wm (drho, j_n, j_t).
+template <int d, int side, bool FORCE, class T>
+__device__ __forceinline__ void wall_change(const StepParams &p, const Coef<float> &cf, const T Fi[3], const T Fo[3],
+                                            const T Fc[3], const T cm[3], T Gcn, T Gct, T wm[3], T dF[3]) {
+    constexpr int wid = 2 * d + side, sg = side == 0 ? 1 : -1;  // sg: the incoming velocities' e_n
+    const float *mw = p.fwm[wid];
+    T mc[2] = {cm[1], cm[2]};  // normal, tangential
+    if constexpr (FORCE) {
+        const T w = all<T>(cf.wface * cf.rho0);
+        mc[0] = fma(Gcn, w, mc[0]);
+        mc[1] = fma(Gct, w, mc[1]);
     }
-    __syncthreads();
-    float fyp[NF];
-#pragma unroll
-    for (int i = 0; i < NF; i++) fyp[i] = 0.0f;
-    if (need_y) {
-        if (!pery && (gy == -1 || gy == ny - 1)) {
-            direct_face(1, gy + 1, fyp);
+    const int type = p.bc[wid];
+    const bool vel = type == 1;
+    const T dra = vel ? cm[0] : all<T>(wall_drho<float>(p, cf, wid));
+    const T man = vel ? all<T>(mw[d]) : mc[0], mat = vel ? all<T>(mw[1 - d]) : mc[1];
+    sfor<3>([&](auto ic) {
+        constexpr int i = ic, t = i - 1;
+        constexpr int k = d == 0 ? 3 * (sg + 1) + t + 1 : 3 * (t + 1) + sg + 1;
+        T v;
+        if (type == 3) {
+            const float em = (float)sg * mw[d] + (float)t * mw[1 - d];
+            v = add(Fo[i], all<T>(wmul<9, float>(k, 6.0f * em)));
         } else {
-            const float *nb = xb + ((row + 1) * 32 + lane) * K::BS;
-            float F[NF], jb[2];
-#pragma unroll
-            for (int i = 0; i < NF; i++) F[i] = aly[i] + nb[i];
-#pragma unroll
-            for (int a = 0; a < 2; a++) jb[a] = Ay[1 + a] + nb[NF + 1 + a];
-            float Gb[2] = {0.0f, 0.0f};
-            if (FORCE) {
-                float G3[3];
-                faceG(1, gx, gy + 1, G3);
-                Gb[0] = G3[0];
-                Gb[1] = G3[1];
-            }
-            face_relax_2d<1, FORCE>(cf, F, Ay[0] + nb[NF], jb, Gb, fyp);
+            const T a = d == 0 ? geq2<k>(cf, dra, man, mat) : geq2<k>(cf, dra, mat, man);
+            const T c = d == 0 ? geq2<k>(cf, cm[0], mc[0], mc[1]) : geq2<k>(cf, cm[0], mc[1], mc[0]);
+            v = add(a, sub(Fc[i], c));
         }
-        float *o = xf + (row * 32 + lane) * K::FS;
+        dF[i] = sub(v, Fi[i]);
+    });
+    const T s = add(add(dF[0], dF[1]), dF[2]);
+    wm[0] = add(wm[0], s);
+    wm[1] = sg > 0 ? add(wm[1], s) : sub(wm[1], s);
+    wm[2] = add(wm[2], sub(dF[2], dF[0]));
+}
+
+// Step 5 of a y wall (side 0: y = 0, 1: y = ny), done by the warp of the ghost row beyond it, which
+// has nothing else to do while the tile's rows form their x interfaces. own: the lane's slots of
+// the ghost row. Into its u0 slots go the wall interface's moments (drho, j_y, j_x) and the changes of
+// the incoming velocities (e_x = -1, 0, 1).
+template <int side, bool FORCE>
+__device__ __forceinline__ void y_wall(const StepParams &p, const Coef<float> &cf, V *own) {
+    constexpr int NS = slots<FORCE>(), dw = side == 0 ? 0 : -1, dc = side == 0 ? 1 : -2;  // low rows of the wall, of x_c
+    const float kap = cf.kappa;
+    auto pub = [&](int dr, int i) __attribute__((always_inline)) -> V & { return own[(dr * NS + i) * 32]; };
+    auto value = [&](int dr, auto kc) __attribute__((always_inline)) -> V {  // step 4, rows dr and dr + 1
+        constexpr int k = decltype(kc)::value;
+        const V l = pub(dr, PF + yi(k)), r = pub(dr + 1, PF + yi(k));
+        V v = fma(bc(-kap * (float)ey(k)), sub(r, l), mul(bc(0.5f), add(l, r)));
+        if constexpr (ex(k) != 0)
+            v = fma(bc(-0.25f * kap * (float)ex(k)), add(pub(dr, PDX + di(k)), pub(dr + 1, PDX + di(k))), v);
+        return v;
+    };
+    V Fi[3], Fo[3], Fc[3], wm[3], cm[3], dF[3], Gc[2] = {bc(0.0f), bc(0.0f)};
+    sfor<3>([&](auto ic) {
+        constexpr int i = ic, k = 3 * i + (side == 0 ? 2 : 0);
+        Fi[i] = value(dw, std::integral_constant<int, k>{});
+        Fo[i] = value(dw, std::integral_constant<int, 8 - k>{});
+        Fc[i] = value(dc, std::integral_constant<int, k>{});
+        wm[i] = add(pub(dw, PA + i), pub(dw + 1, PB + i));
+        cm[i] = add(pub(dc, PA + i), pub(dc + 1, PB + i));
+    });
+    if constexpr (FORCE) {
 #pragma unroll
-        for (int i = 0; i < NF; i++) o[i] = fyp[i];
+        for (int c = 0; c < 2; c++)
+            Gc[c] = mul(add(bc(p.fg[c]), mul(bc(0.5f), add(pub(dc, PFLD + c), pub(dc + 1, PFLD + c)))), bc(cf.cth));
+    }
+    wall_change<1, side, FORCE>(p, cf, Fi, Fo, Fc, cm, Gc[1], Gc[0], wm, dF);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        pub(0, PU + i) = wm[i];
+        pub(0, PU + 3 + i) = dF[i];
+    }
+}
+
+// Step 5 for the columns at x walls (own: the lane's slots of its row): column 0's -x and column
+// nx - 1's +x interface. Both walls' lanes run the same code at once, with the side (sg: the incoming
+// velocities' e_x) as data.
+struct XWall {
+    V fe[3], fw[3], Ge[2], Gw[2];  // in/out: moments at the columns' x interfaces; in: G there (n, t)
+    V lo[3], hi[3];                // out: changes at column 0's -x and column nx - 1's +x interface
+};
+template <bool FORCE>
+__device__ __forceinline__ void x_wall(const StepParams &p, const Coef<float> &cf, const Strip &s, const V *own, XWall &w) {
+    constexpr int NS = slots<FORCE>();
+    const float kap = cf.kappa, ir = cf.inv_rho0;
+    auto pub = [&](int dr, int i) __attribute__((always_inline)) -> const V & { return own[(dr * NS + i) * 32]; };
+    // step-4 values of the six crossing velocities at the +x interface of every column
+    V F[9];
+    sfor<9>([&](auto kc) {
+        constexpr int k = kc;
+        if constexpr (ex(k) != 0) {
+            const V l = pub(0, ey(k) != 0 ? PF + yi(k) : PX + k / 7), r = east(l);
+            V v = fma(bc(-kap * (float)ex(k)), sub(r, l), mul(bc(0.5f), add(l, r)));
+            if constexpr (ey(k) != 0) {
+                const V C = sub(pub(1, PF + yi(k)), pub(-1, PF + yi(k)));
+                v = fma(bc(-0.25f * kap * (float)ey(k)), add(C, east(C)), v);
+            }
+            F[k] = v;
+        }
+    });
+#pragma unroll
+    for (int i = 0; i < 3; i++) w.lo[i] = w.hi[i] = bc(0.0f);
+    const bool at0 = s.gx0 == p.nx - 1, at1 = s.gx0 + 1 == p.nx - 1;
+    bool lo = s.xlo && s.gx0 == 0, hi = s.xhi && (at0 || at1);
+    // a lane with both walls (nx = 2) takes a second pass
+    for (bool both = __any_sync(0xffffffffu, lo && hi);; both = false) {
+        const bool l = lo;
+        const float sg = l ? 1.0f : -1.0f;
+        const int wid = l ? 0 : 1, type = p.bc[wid];
+        // the wall's and x_c's values: column 0's -x and +x interfaces, column nx - 1's +x and -x ones
+        auto pick = [&](V e, V we, bool wall) __attribute__((always_inline)) {
+            const V v = wall == l ? we : e;
+            return l || at0 ? v.x : v.y;
+        };
+        float Fi[3], Fo[3], Fc[3], cm[3], wm[3], Gc[2];
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const V a = F[i], b = F[6 + i], wa = west(a), wb = west(b);  // e_x = -1, +1 with e_y = i - 1
+            Fi[i] = l ? pick(b, wb, true) : pick(a, wa, true);
+            Fc[i] = l ? pick(b, wb, false) : pick(a, wa, false);
+            const V oa = F[2 - i], ob = F[8 - i], woa = west(oa), wob = west(ob);  // the opposites
+            Fo[i] = l ? pick(oa, woa, true) : pick(ob, wob, true);
+            wm[i] = pick(w.fe[i], w.fw[i], true);
+            cm[i] = pick(w.fe[i], w.fw[i], false);
+        }
+#pragma unroll
+        for (int c = 0; c < 2; c++) Gc[c] = pick(w.Ge[c], w.Gw[c], false);
+        if (lo || hi) {
+            const float *mw = p.fwm[wid];
+            float mc[2] = {cm[1], cm[2]};
+            if constexpr (FORCE) {
+                mc[0] = fmaf(Gc[0], cf.wface * cf.rho0, mc[0]);
+                mc[1] = fmaf(Gc[1], cf.wface * cf.rho0, mc[1]);
+            }
+            const bool vel = type == 1;
+            const float dra = vel ? cm[0] : wall_drho<float>(p, cf, wid);
+            const float ma[2] = {vel ? mw[0] : mc[0], vel ? mw[1] : mc[1]};
+            const float ba = fmaf(-1.5f * ir, fmaf(ma[0], ma[0], ma[1] * ma[1]), dra);
+            const float bcc = fmaf(-1.5f * ir, fmaf(mc[0], mc[0], mc[1] * mc[1]), cm[0]);
+            float d[3], sum = 0.0f;
+            sfor<3>([&](auto ic) {
+                constexpr int i = ic, t = i - 1;
+                constexpr double W = t == 0 ? 1.0 / 9.0 : 1.0 / 36.0;
+                constexpr float wh = (float)W, wl = (float)(W - (double)wh);
+                auto geq = [&](const float *m, float b) __attribute__((always_inline)) {
+                    const float em = fmaf((float)t, m[1], sg * m[0]);
+                    const float x = fmaf(em, 3.0f, fmaf(ir * em, 4.5f * em, b));
+                    return fmaf(wl, x, wh * x);
+                };
+                const float em6 = 6.0f * (sg * mw[0] + (float)t * mw[1]);
+                const float v = type == 3 ? Fo[i] + fmaf(wl, em6, wh * em6) : geq(ma, ba) + (Fc[i] - geq(mc, bcc));
+                d[i] = v - Fi[i];
+                sum += d[i];
+            });
+            wm[0] += sum;
+            wm[1] = fmaf(sg, sum, wm[1]);
+            wm[2] += d[2] - d[0];
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                if (l) { w.fw[i].x = wm[i]; w.lo[i].x = d[i]; }
+                else if (at0) { w.fe[i].x = wm[i]; w.hi[i].x = d[i]; }
+                else { w.fe[i].y = wm[i]; w.hi[i].y = d[i]; }
+            }
+        }
+        if (!both) break;
+        hi = lo && hi;  // the second pass: the lanes whose other wall is left
+        lo = false;
+    }
+}
+
+// With a force it is kept out of line: inlined, the tile spills at 80 registers.
+template <bool FORCE>
+__device__ __noinline__ void x_wall_call(const StepParams &p, const Strip s, const V *own, XWall &w) {
+    const Coef<float> cf(p);
+    x_wall<FORCE>(p, cf, s, own, w);
+}
+
+// One tile: columns [x0, x0 + 60) x rows [y0, y0 + RY - 2) of the instance p, by a block of 32 x RY
+// threads; sm: smem_bytes(RY). Called by every thread of the block.
+template <class S, bool FORCE>
+__device__ __forceinline__ void tile(const StepParams &p, V *sm, int x0, int y0) {
+    constexpr int NN = FORCE ? 6 : 5, NS = slots<FORCE>();
+    const Coef<float> cf(p);
+    const Strip s = make_strip(p, x0);
+    const int ny = p.ny, ry = blockDim.y, row = threadIdx.y, gy = y0 - 1 + row;
+    const bool pery = p.bc[2] == 0;
+    const float kap = cf.kappa;
+    V *own = sm + row * NS * 32 + s.lane;  // this row's published values
+    auto pub = [&](int dr, int i) __attribute__((always_inline)) -> V & { return own[(dr * NS + i) * 32]; };
+    const bool real = (gy >= 0 && gy < ny) || (pery && gy >= -1 && gy <= ny);
+    const bool upd = row >= 1 && row <= ry - 2 && gy < ny;
+    const V ca = bc(0.5f - kap), cb = bc(0.5f + kap), ch = bc(0.5f * kap), cn = bc(-0.5f * kap);
+
+    uint32_t seed = 0;  // stochastic rounding of F16 stores
+    if constexpr (sizeof(S) == 2) seed = store_seed(*p.step_ctr + p.step_off);
+
+    // ---- step 1 and what needs the own row only: La's x part, the y interfaces' parts ----
+    Row n;
+    V La[9];
+    if (real) {
+        const int y = wrap_idx(gy, ny);
+        {
+            V g[9], u0[9];
+            load_row<S>(p, s, y, g);
+            make_row<FORCE>(p, cf, s, y, g, n, u0);
+#pragma unroll
+            for (int k = 0; k < 9; k++) pub(0, PU + k) = u0[k];
+        }
+        sfor<9>([&](auto kc) {
+            constexpr int k = kc;
+            if constexpr (ex(k) != 0) {
+                const V e = east(n.f[k]), w = west(n.f[k]);
+                const V dE = ex(k) > 0 ? sub(e, n.f[k]) : sub(n.f[k], e);
+                const V dW = ex(k) > 0 ? sub(n.f[k], w) : sub(w, n.f[k]);
+                La[k] = fma(ex(k) > 0 ? ca : cb, dE, mul(ex(k) > 0 ? cb : ca, dW));
+                if constexpr (ey(k) != 0) pub(0, PDX + di(k)) = sub(e, w);
+            }
+            if constexpr (ey(k) != 0) pub(0, PF + yi(k)) = n.f[k];
+            else if constexpr (k != 4) pub(0, PX + k / 7) = n.f[k];
+        });
+        V Dx[3], A[3];
+        x_diffs(n.m, Dx);
+        moment_parts<1>(kap, n.m[0], n.m[2], n.m[1], n.m[4], n.m[5], Dx, A);
+#pragma unroll
+        for (int i = 0; i < 3; i++) pub(0, PA + i) = A[i];
+        moment_parts<-1>(kap, n.m[0], n.m[2], n.m[1], n.m[4], n.m[5], Dx, A);
+#pragma unroll
+        for (int i = 0; i < 3; i++) pub(0, PB + i) = A[i];
+        pub(0, PM) = n.m[2];
+        pub(0, PM + 1) = n.m[5];
+        pub(0, PM + 2) = n.m[4];
+        if constexpr (FORCE) {
+            pub(0, PFLD) = n.fld[0];
+            pub(0, PFLD + 1) = n.fld[1];
+        }
+    }
+    const bool ywalls = !pery && (y0 == 0 || y0 + ry - 2 >= ny);  // the tile holds a ghost row
+    const bool ghost = ywalls && (gy == -1 || gy == ny);
+    if (ywalls) {
+        __syncthreads();
+        if (ghost) {  // step 2: 2 f0 - f1
+            const int d = gy < 0 ? 1 : -1;
+            for (int i = 0; i < PX; i++) {
+                const V a = pub(d, i);
+                pub(0, i) = sub(add(a, a), pub(2 * d, i));
+            }
+            if constexpr (FORCE) {  // a wall interface takes the one adjacent cell's acceleration
+                pub(0, PFLD) = pub(d, PFLD);
+                pub(0, PFLD + 1) = pub(d, PFLD + 1);
+            }
+        }
     }
     __syncthreads();
 
-    // ---- steps 8-9: update of the own cell ----
-    float fxm[NF];
-    if (row >= 1 && row <= K::TYI) {
+    // from here on the row's own fbar+ is read back where it is needed: the registers hold La and M0,
+    // M_x, M_xx
+    // acceleration / c at an interface: mean of the two cells (reading R2)
+    auto mean = [&](int c, V a, V b) __attribute__((always_inline)) -> V {
+        if constexpr (FORCE) return mul(add(bc(p.fg[c]), mul(bc(0.5f), add(a, b))), bc(cf.cth));
+        else return bc(0.0f);
+    };
+    auto fld = [&](int dr, int c) __attribute__((always_inline)) -> V {
+        if constexpr (FORCE) return pub(dr, PFLD + c);
+        else return bc(0.0f);
+    };
+    V X[6], Y[6];  // differences of the interfaces' numbers: x (E - W), y (N - S)
+    if (upd) {  // warp-uniform
+        // ---- x interfaces (E, W): parts exchanged by shuffles ----
+        V fe[3], fw[3], Ge[2], Gw[2];
+        {
+            V D[3], A[3], B[3];
+            D[0] = sub(pub(1, PM), pub(-1, PM));
+            D[1] = sub(pub(1, PM + 1), pub(-1, PM + 1));
+            D[2] = sub(pub(1, PM + 2), pub(-1, PM + 2));
+            const V my = pub(0, PM), mxy = pub(0, PM + 1);
+            moment_parts<1>(kap, n.m[0], n.m[1], my, n.m[3], mxy, D, A);
+            moment_parts<-1>(kap, n.m[0], n.m[1], my, n.m[3], mxy, D, B);
 #pragma unroll
-        for (int i = 0; i < NF; i++) fxm[i] = __shfl_up_sync(0xffffffffu, fxp[i], 1);
+            for (int i = 0; i < 3; i++) {
+                fe[i] = add(A[i], east(B[i]));
+                fw[i] = add(west(A[i]), B[i]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            Ge[c] = mean(c, fld(0, c), FORCE ? east(fld(0, c)) : fld(0, c));
+            Gw[c] = mean(c, FORCE ? west(fld(0, c)) : fld(0, c), fld(0, c));
+        }
+        if (s.xlo || s.xhi) {  // step 5 at x walls
+            XWall w;
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                w.fe[i] = fe[i];
+                w.fw[i] = fw[i];
+            }
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                w.Ge[c] = Ge[c];
+                w.Gw[c] = Gw[c];
+            }
+            if constexpr (FORCE) x_wall_call<FORCE>(p, s, own, w);
+            else x_wall<FORCE>(p, cf, s, own, w);
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                fe[i] = w.fe[i];
+                fw[i] = w.fw[i];
+                La[i] = sub(La[i], w.hi[i]);
+                La[6 + i] = sub(La[6 + i], w.lo[i]);
+            }
+        }
+        {
+            V a[6], b[6];
+            face_numbers<FORCE>(cf, fe, Ge[0], Ge[1], a);
+            face_numbers<FORCE>(cf, fw, Gw[0], Gw[1], b);
+#pragma unroll
+            for (int i = 0; i < NN; i++) X[i] = sub(a[i], b[i]);
+        }
+    } else if (ghost) {
+        if (gy < 0) y_wall<0, FORCE>(p, cf, own);
+        else y_wall<1, FORCE>(p, cf, own);
     }
-    if (upd) {
-        const float *ym = xf + ((row - 1) * 32 + lane) * K::FS;
-        const int64_t off = (int64_t)gy * p.px + gx;
+    if (ywalls) __syncthreads();
+    if (!upd) return;
+    // ---- y interfaces (N, S): moments from the parts of the two rows ----
+    V fn[3], fs[3], Gn[2], Gs[2];
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        fn[i] = add(pub(0, PA + i), pub(1, PB + i));
+        fs[i] = add(pub(-1, PA + i), pub(0, PB + i));
+    }
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        Gn[c] = mean(c, fld(0, c), fld(1, c));
+        Gs[c] = mean(c, fld(-1, c), fld(0, c));
+    }
+    // La's y part and the mixed differences
+    sfor<9>([&](auto kc) {
+        constexpr int k = kc;
+        if constexpr (ey(k) != 0) {
+            const V f = pub(0, PF + yi(k)), N = pub(1, PF + yi(k)), Sv = pub(-1, PF + yi(k));
+            const V dN = ey(k) > 0 ? sub(N, f) : sub(f, N), dS = ey(k) > 0 ? sub(f, Sv) : sub(Sv, f);
+            V l = mul(ey(k) > 0 ? cb : ca, dS);
+            if constexpr (ex(k) != 0) {
+                l = add(La[k], l);
+                l = fma(ex(k) * ey(k) > 0 ? ch : cn, sub(pub(-1, PDX + di(k)), pub(1, PDX + di(k))), l);
+            }
+            La[k] = fma(ey(k) > 0 ? ca : cb, dN, l);
+        }
+    });
+    // step 5 at y walls: the changes of the incoming velocities enter La and the moments
+    if (ywalls && gy == 0) {
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            fs[i] = pub(-1, PU + i);
+            La[3 * i + 2] = sub(La[3 * i + 2], pub(-1, PU + 3 + i));
+        }
+    }
+    if (ywalls && gy == ny - 1) {
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            fn[i] = pub(1, PU + i);
+            La[3 * i] = sub(La[3 * i], pub(1, PU + 3 + i));
+        }
+    }
+    {
+        V a[6], b[6];
+        face_numbers<FORCE>(cf, fn, Gn[1], Gn[0], a);
+        face_numbers<FORCE>(cf, fs, Gs[1], Gs[0], b);
+#pragma unroll
+        for (int i = 0; i < NN; i++) Y[i] = sub(a[i], b[i]);
+    }
+    // ---- step 8 ----
+    V N[9];
+    const V zero = bc(0.0f);
+    if constexpr (FORCE) {
+        N[7] = X[0];
+        N[1] = sub(zero, X[1]);
+        N[5] = Y[0];
+        N[3] = sub(zero, Y[1]);
+        N[8] = add(X[2], Y[2]);
+        N[0] = sub(zero, add(X[3], Y[3]));
+        N[6] = sub(X[4], Y[5]);
+        N[2] = sub(Y[4], X[5]);
+    } else {
+        const V t3 = bc(3.0f), x3 = mul(t3, X[3]), y3 = mul(t3, Y[3]);
+        N[7] = add(x3, X[0]);
+        N[1] = sub(x3, X[0]);
+        N[5] = add(y3, Y[0]);
+        N[3] = sub(y3, Y[0]);
+        const V o1 = add(X[1], Y[2]), o2 = add(X[2], Y[1]);
+        const V e1 = add(x3, y3), e2 = mul(t3, add(X[4], Y[4]));
+        const V op = add(o1, o2), om = sub(o1, o2), ep = add(e1, e2), em = sub(e1, e2);
+        N[8] = add(ep, op);
+        N[0] = sub(ep, op);
+        N[6] = add(em, om);
+        N[2] = sub(em, om);
+    }
+    // ---- step 9, eq. (16) ----
+    const float tk = -cf.two_kappa * (FORCE ? 1.0f : cf.b7);
+    const V cL = bc(-cf.two_kappa * (1.0f - cf.b7)), w1 = bc(tk * (1.0f / 9.0f)), w2 = bc(tk * (1.0f / 36.0f));
+    V u0[9];
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        u0[k] = pub(0, PU + k);
+        if (k != 4) u0[k] = add(u0[k], fma(ex(k) != 0 && ey(k) != 0 ? w2 : w1, N[k], mul(cL, La[k])));
+    }
+    const bool mine = s.lane >= 1 && s.lane <= TXI / 2;
+    const bool upd0 = mine && s.gx0 < p.nx, upd1 = mine && s.gx0 + 1 < p.nx;
+    const int64_t off = (int64_t)gy * p.px + s.gx0;
+    S *o = reinterpret_cast<S *>(p.dst) + off;
+    if constexpr (sizeof(S) == 4) {
+        if (upd1) {
+#pragma unroll
+            for (int k = 0; k < 9; k++) *reinterpret_cast<float2 *>(o + k * p.dstride) = u0[k];
+        } else if (upd0) {
+#pragma unroll
+            for (int k = 0; k < 9; k++) o[k * p.dstride] = u0[k].x;
+        }
+    } else {
+        // F16: one conversion rounds the lane's two cells stochastically, fed by one random word (some
+        // 150 instructions less than rounding each in software)
         const CellRandom rnd(seed, off);
-        sfor<Q>([&](auto kc) {
+        sfor<9>([&](auto kc) {
             constexpr int k = kc;
-            float acc = 0.0f;
-            if constexpr (Lat<9>::e(k, 0) != 0) {
-                constexpr int i = flux_index<9>(0, k);
-                acc = fmaf((float)Lat<9>::e(k, 0), fxp[i] - fxm[i], acc);
-            }
-            if constexpr (Lat<9>::e(k, 1) != 0) {
-                constexpr int i = flux_index<9>(1, k);
-                acc = fmaf((float)Lat<9>::e(k, 1), fyp[i] - ym[i], acc);
-            }
-            // eq. (25) in increment form (4/3 fbar+ - 1/3 f~), then the flux of
-            // eq. (16)
-            const float u0 = fmaf(1.0f / 3.0f, f[k] - g[k], f[k]);
-            store_state<S>(dst + k * p.dstride + off, fmaf(-cf.two_kappa, acc, u0), sizeof(S) == 2 ? rnd.bits<k>() : 0u);
+            const uint32_t w = f16_pair(u0[k], rnd.template word<k>());
+            if (upd1) *reinterpret_cast<uint32_t *>(o + k * p.dstride) = w;
+            else if (upd0) o[k * p.dstride] = __ushort_as_half((unsigned short)(w & 0xffffu));
         });
     }
 }
 
-template <class S, int RY, bool FORCE>
-__global__ void __launch_bounds__(32 * RY) fused_step2d(const __grid_constant__ StepParams p) {
-    using K = Shape2<RY, S>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    step2d_tile<S, RY, FORCE>(p, smem_raw, blockIdx.x * K::TXI, blockIdx.y * K::TYI);
+}  // namespace m2
+
+// One instance on a grid of tiles.
+template <class S, bool FORCE>
+__global__ void __launch_bounds__(m2::REG_THREADS) fused_step2d(const __grid_constant__ StepParams p) {
+    extern __shared__ __align__(16) float2 smem2[];
+    chain_wait();
+    m2::tile<S, FORCE>(p, smem2, blockIdx.x * m2::TXI, blockIdx.y * (blockDim.y - 2));
 }
 
 // Batched form: params holds two descriptors per instance (source/destination swapped:
-// index 2 i + parity); items is the work list of (instance, x0, y0, -) inner-tile origins,
-// largest instances first; CTA b takes items b, b + gridDim.x, ...
-template <class S, int RY, bool FORCE>
-__global__ void __launch_bounds__(32 * RY) fused_step2d_batch(const StepParams *__restrict__ params,
-                                                              const int4 *__restrict__ items, int nitems, int parity) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+// index 2 i + parity); items is the work list of (instance, x0, y0, -) tiles, largest
+// instances first; block b takes items b, b + gridDim.x, ... Each instance takes the path with
+// or without the force term that it would take alone: FORCE 0 none of them has a force, 1 all
+// have (both with the registers of their one path), 2 some.
+template <class S, int FORCE>
+__global__ void __launch_bounds__(m2::REG_THREADS) fused_step2d_batch(const StepParams *__restrict__ params,
+                                                                    const int4 *__restrict__ items, int nitems,
+                                                                    int parity) {
+    extern __shared__ __align__(16) float2 smem2[];
+    __shared__ __align__(16) StepParams p;
+    chain_wait();
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 w = items[it];
-        step2d_tile<S, RY, FORCE>(params[2 * w.x + parity], smem_raw, w.y, w.z);
-        __syncthreads();  // the next item reuses the shared buffers
+        {  // the instance's parameters, as the constant bank holds them for one instance
+            const uint32_t *q = reinterpret_cast<const uint32_t *>(params + 2 * w.x + parity);
+            for (int i = threadIdx.y * 32 + threadIdx.x; i < (int)(sizeof(StepParams) / 4); i += 32 * blockDim.y)
+                reinterpret_cast<uint32_t *>(&p)[i] = __ldg(q + i);
+        }
+        __syncthreads();
+        if constexpr (FORCE != 2) {
+            m2::tile<S, FORCE != 0>(p, smem2, w.y, w.z);
+        } else {
+            if (p.field != nullptr || p.g[0] != 0.0 || p.g[1] != 0.0) m2::tile<S, true>(p, smem2, w.y, w.z);
+            else m2::tile<S, false>(p, smem2, w.y, w.z);
+        }
+        __syncthreads();  // the next item reuses the shared memory
     }
 }
 

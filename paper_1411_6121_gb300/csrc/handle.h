@@ -57,7 +57,7 @@ struct dugks_s {
     double *d_metric;      // non-uniform mesh metrics (device; NULL: uniform), see StepParams
     double eg[3][2];       // its ghost extrapolation coefficients
     int64_t metric_off[3]; // offset of each axis' block in d_metric
-    int ry3d;              // CTA rows of the 3D throughput kernel
+    int ry3d;              // CTA rows of the throughput kernels (0: the default form)
     int own_stream;
     size_t esize;          // bytes per stored element
     size_t state_bytes;    // padded device bytes of one buffer

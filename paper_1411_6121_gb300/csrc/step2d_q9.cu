@@ -1,5 +1,7 @@
 // step2d_q9.cu -- instantiations and launchers of the D2Q9 throughput kernel
 // (dugks_step2d.cuh): one instance on a grid of tiles, or a batch on a persistent grid.
+#include <algorithm>
+
 #include "dugks_internal.h"
 #include "dugks_step2d.cuh"
 
@@ -7,98 +9,108 @@ namespace dugks {
 
 namespace {
 
-template <class S, int RY, bool FORCE, bool BATCH>
-cudaError_t configure(int *blocks_per_sm, int *sms) {
-    using K = Shape2<RY, S>;
-    static int configured_dev = -1;
-    static int cached_bps = 0, cached_sms = 0;
+// Resident blocks per SM of a kernel at every number of block rows, for one device.
+struct Residency {
+    int dev = -1, sms = 1, blocks[m2::MAX_RY + 1] = {};
+};
+
+// FORCE: as the batch kernel's; the single kernel has 0 and 1.
+template <class S, int FORCE, bool BATCH>
+cudaError_t configure(const Residency **out) {
+    static Residency r;
     int dev = 0;
     cudaGetDevice(&dev);
-    if (configured_dev != dev) {
-        cudaError_t e;
-        if (BATCH)
-            e = cudaFuncSetAttribute(fused_step2d_batch<S, RY, FORCE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)K::smem_bytes);
-        else
-            e = cudaFuncSetAttribute(fused_step2d<S, RY, FORCE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)K::smem_bytes);
+    if (r.dev != dev) {
+        const void *fn;
+        if constexpr (BATCH) fn = (const void *)fused_step2d_batch<S, FORCE>;
+        else fn = (const void *)fused_step2d<S, FORCE != 0>;
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)m2::smem_bytes<FORCE != 0>(m2::MAX_RY));
         if (e != cudaSuccess) return e;
-        if (BATCH)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cached_bps, fused_step2d_batch<S, RY, FORCE>, 32 * RY,
-                                                          K::smem_bytes);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cached_bps, fused_step2d<S, RY, FORCE>, 32 * RY,
-                                                          K::smem_bytes);
-        cudaDeviceGetAttribute(&cached_sms, cudaDevAttrMultiProcessorCount, dev);
-        configured_dev = dev;
+        for (int ry = 3; ry <= m2::MAX_RY; ry++) {
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.blocks[ry], fn, 32 * ry, m2::smem_bytes<FORCE != 0>(ry));
+            r.blocks[ry] = std::max(1, r.blocks[ry]);
+        }
+        cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev);
+        r.dev = dev;
     }
-    if (blocks_per_sm) *blocks_per_sm = cached_bps < 1 ? 1 : cached_bps;
-    if (sms) *sms = cached_sms;
+    *out = &r;
     return cudaSuccess;
 }
 
-template <class S, int RY, bool FORCE>
-cudaError_t launch_one(const StepParams &p, cudaStream_t stream) {
-    using K = Shape2<RY, S>;
-    cudaError_t e = configure<S, RY, FORCE, false>(nullptr, nullptr);
-    if (e != cudaSuccess) return e;
-    dim3 grid((p.nx + K::TXI - 1) / K::TXI, (p.ny + K::TYI - 1) / K::TYI);
-    fused_step2d<S, RY, FORCE><<<grid, dim3(32, RY), K::smem_bytes, stream>>>(p);
-    return cudaGetLastError();
+// Block rows of an nx x ny mesh: the ones that leave the busiest SM the fewest warps to run,
+// counted against 24 resident ones where they come in waves (10 and 16 rows fit 20 and 16 per
+// SM); the smaller block on a tie. A block updates ry - 2 of its rows, so large meshes take 12 rows
+// and small ones, where a step is the latency of one block, few. us per step with 4 / 6 / 8 / 12
+// rows: 128 x 64 channel 3.38 / 3.72 / 4.04 / 5.01, 512 x 256 channel 7.64 / 6.70 / 7.05 / 7.04, 2048^2
+// cavity 124 / 106 / 103 / 102.
+int block_rows(int64_t nx, int64_t ny, const Residency &r) {
+    const int64_t strips = (nx + m2::TXI - 1) / m2::TXI;
+    const int cand[] = {3, 4, 6, 8, 12};
+    int best = 8;
+    double least = 1e300;
+    for (int ry : cand) {
+        const int64_t blocks = strips * ((ny + ry - 3) / (ry - 2));
+        const double warps = (double)((blocks + r.sms - 1) / r.sms) * ry;
+        const int cap = std::min(24, r.blocks[ry] * ry);
+        const double cost = warps > cap ? warps * 24.0 / cap : warps;
+        if (cost < least) {
+            least = cost;
+            best = ry;
+        }
+    }
+    return best;
 }
 
-template <class S, int RY, bool FORCE>
-cudaError_t launch_many(const StepParams *params, const int4 *items, int nitems, int parity, cudaStream_t stream) {
-    using K = Shape2<RY, S>;
-    int bps = 1, sms = 1;
-    cudaError_t e = configure<S, RY, FORCE, true>(&bps, &sms);
+template <class S, bool FORCE>
+cudaError_t launch_one(const StepParams &p, int ry, cudaStream_t stream) {
+    const Residency *r;
+    cudaError_t e = configure<S, FORCE, false>(&r);
     if (e != cudaSuccess) return e;
-    const int grid = nitems < sms * bps ? nitems : sms * bps;  // persistent: resident CTAs, at most the items
+    if (ry == 0) ry = block_rows(p.nx, p.ny, *r);
+    const dim3 grid((p.nx + m2::TXI - 1) / m2::TXI, (p.ny + ry - 3) / (ry - 2));
+    return launch_chained(fused_step2d<S, FORCE>, grid, dim3(32, ry), m2::smem_bytes<FORCE>(ry), stream, p);
+}
+
+template <class S, int FORCE>
+cudaError_t launch_many(const StepParams *params, const int4 *items, int nitems, int parity, int ry,
+                        cudaStream_t stream) {
+    const Residency *r;
+    cudaError_t e = configure<S, FORCE, true>(&r);
+    if (e != cudaSuccess) return e;
+    const int grid = std::min(nitems, r->sms * r->blocks[ry]);  // persistent: the resident blocks, at most the items
     if (grid < 1) return cudaSuccess;
-    fused_step2d_batch<S, RY, FORCE><<<grid, dim3(32, RY), K::smem_bytes, stream>>>(params, items, nitems, parity);
-    return cudaGetLastError();
+    return launch_chained(fused_step2d_batch<S, FORCE>, dim3(grid), dim3(32, ry), m2::smem_bytes<FORCE != 0>(ry), stream,
+                          params, items, nitems, parity);
 }
 
-template <class S, bool FORCE>
-cudaError_t one_ry(const StepParams &p, int ry, cudaStream_t st) {
-    if (ry == 4) return launch_one<S, 4, FORCE>(p, st);
-    if (ry == 8) return launch_one<S, 8, FORCE>(p, st);
-    if (ry == 16) return launch_one<S, 16, FORCE>(p, st);
-    return cudaErrorNotSupported;
-}
-
-template <class S, bool FORCE>
-cudaError_t many_ry(const StepParams *params, const int4 *items, int nitems, int parity, int ry, cudaStream_t st) {
-    if (ry == 4) return launch_many<S, 4, FORCE>(params, items, nitems, parity, st);
-    if (ry == 8) return launch_many<S, 8, FORCE>(params, items, nitems, parity, st);
-    if (ry == 16) return launch_many<S, 16, FORCE>(params, items, nitems, parity, st);
-    return cudaErrorNotSupported;
+template <class S>
+cudaError_t many(const StepParams *params, const int4 *items, int nitems, int parity, int ry, int force, cudaStream_t st) {
+    if (force == 0) return launch_many<S, 0>(params, items, nitems, parity, ry, st);
+    if (force == 1) return launch_many<S, 1>(params, items, nitems, parity, ry, st);
+    return launch_many<S, 2>(params, items, nitems, parity, ry, st);
 }
 
 }  // namespace
 
+int step2d_tile_columns(int store) { return store == 1 ? 30 : m2::TXI; }
+
 cudaError_t launch_step2d_q9(const StepParams &p, int store, int ry, cudaStream_t stream) {
     const bool force = p.field != nullptr || p.g[0] != 0.0 || p.g[1] != 0.0;
     switch (store) {
-        case 0: return force ? one_ry<float, true>(p, ry, stream) : one_ry<float, false>(p, ry, stream);
-        case 1: return force ? one_ry<__nv_bfloat16, true>(p, ry, stream) : one_ry<__nv_bfloat16, false>(p, ry, stream);
-        case 2: return force ? one_ry<__half, true>(p, ry, stream) : one_ry<__half, false>(p, ry, stream);
+        case 0: return force ? launch_one<float, true>(p, ry, stream) : launch_one<float, false>(p, ry, stream);
+        case 1: return launch_step2d_q9_bf16(p, ry, stream);
+        case 2: return force ? launch_one<__half, true>(p, ry, stream) : launch_one<__half, false>(p, ry, stream);
     }
     return cudaErrorNotSupported;
 }
 
 cudaError_t launch_step2d_batch(const StepParams *params, const int4 *items, int nitems, int parity, int store,
-                                int ry, bool force, cudaStream_t stream) {
+                                int ry, int force, cudaStream_t stream) {
     switch (store) {
-        case 0:
-            return force ? many_ry<float, true>(params, items, nitems, parity, ry, stream)
-                         : many_ry<float, false>(params, items, nitems, parity, ry, stream);
-        case 1:
-            return force ? many_ry<__nv_bfloat16, true>(params, items, nitems, parity, ry, stream)
-                         : many_ry<__nv_bfloat16, false>(params, items, nitems, parity, ry, stream);
-        case 2:
-            return force ? many_ry<__half, true>(params, items, nitems, parity, ry, stream)
-                         : many_ry<__half, false>(params, items, nitems, parity, ry, stream);
+        case 0: return many<float>(params, items, nitems, parity, ry, force, stream);
+        case 1: return launch_step2d_batch_bf16(params, items, nitems, parity, ry, force != 0, stream);
+        case 2: return many<__half>(params, items, nitems, parity, ry, force, stream);
     }
     return cudaErrorNotSupported;
 }

@@ -1,0 +1,70 @@
+"""The 2D step kernels at the edges of their tiles, element by element against the oracle: sizes one
+below, at and one above the columns and rows of a tile, odd sizes (the last column alone in its
+lane), every wall type on both axes, with and without a force; and the same bits whatever the
+block's rows."""
+import numpy as np
+import pytest
+
+from oracle import Oracle
+from paper_1411_6121_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+FLOWS = {
+    "channel": dict(bcs=W.channel_bcs(2), g=(1e-4, -2e-5, 0.0)),
+    "cavity": dict(bcs=W.cavity_bcs(2, 0.1)),
+    "box": dict(bcs=[W.pressure(1e-3), W.wall((0.0, 0.02)), W.bounce_back((0.03, 0.0)), W.bounce_back()], g=(0.0, 1e-4, 0.0)),
+    "periodic": dict(bcs=W.all_periodic()),
+}
+SIZES = [(2, 2), (3, 5), (59, 6), (60, 7), (61, 13), (62, 2), (121, 3)]
+
+
+def _state(o):
+    _, Wt = o.lattice()
+    return o.get_state() - Wt[:, None] * o.cfg.rho0
+
+
+def _pair(cfg, steps, **kw):
+    from paper_1411_6121_gb300 import dugks
+    p, u = W.random_state_fields(cfg["shape"], seed=sum(cfg["shape"]), u_amp=0.03, p_amp=1e-3)
+    o = Oracle(**cfg)
+    o.init(p=p, u=u)
+    o.step(steps)
+    s = dugks.Sim(**cfg, **kw)
+    s.init(p=p, u=u)
+    s.step(steps)
+    return _state(o), s.get_state().astype(np.float64)
+
+
+@pytest.mark.parametrize("flow", sorted(FLOWS))
+@pytest.mark.parametrize("shape", SIZES)
+def test_d2q9_tile_edges(shape, flow):
+    cfg = dict(shape=shape, q=9, nu=0.05, dt=0.5, **FLOWS[flow])
+    ref, got = _pair(cfg, 10)
+    assert np.abs(got - ref).max() < 2e-6 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("flow", ["box", "channel"])
+def test_d2q9_bits_do_not_depend_on_the_block(flow):
+    cfg = dict(shape=(67, 31), q=9, nu=0.05, dt=0.5, **FLOWS[flow])
+    outs = [_pair(cfg, 8, **kw)[1] for kw in ({}, dict(tile=(32, 4)), dict(tile=(32, 8)), dict(tile=(32, 16)))]
+    for o in outs[1:]:
+        assert np.array_equal(o, outs[0])
+
+
+@pytest.mark.parametrize("shape", [(61, 7), (9, 33)])
+def test_d2q9_f16_one_step(shape):
+    """One step from the same stored state: within one stored rounding (2^-10) of the FP64 step."""
+    from paper_1411_6121_gb300 import dugks
+    cfg = dict(shape=shape, q=9, nu=0.05, dt=0.5, **FLOWS["box"])
+    p, u = W.random_state_fields(shape, seed=3, u_amp=0.03, p_amp=1e-3)
+    s = dugks.Sim(store=2, **cfg)
+    s.init(p=p, u=u)
+    g0 = s.get_state().astype(np.float64) / 4096.0
+    o = Oracle(**cfg)
+    _, Wt = o.lattice()
+    o.set_state(g0 + Wt[:, None] * o.cfg.rho0)
+    o.step(1)
+    s.step(1)
+    ref, got = _state(o), s.get_state().astype(np.float64) / 4096.0
+    assert np.all(np.abs(got - ref) <= 2e-6 * np.abs(ref).max() + 2.0 ** -10 * np.abs(ref))
