@@ -124,7 +124,8 @@ typedef struct {
     int32_t tile_x, tile_y; /* 0: default tile. Throughput kernels (kernel 0, F32/BF16/F16
                                storage): tile_y = thread-block rows (D2Q9: 4, 8 or 16, by
                                default chosen by the mesh, with the same results;
-                               D3Q19: 8 or 10; D3Q27: 8; default 8), tile_x ignored.
+                               D3Q19: 8 or 10, D3Q27: 8 take the non-specialised
+                               kernel; default the warp-specialised one), tile_x ignored.
                                Reference
                                kernel: tile_x x tile_y = 32x8 or 16x8                   */
     int32_t kernel;         /* 0: fastest kernel built for the case (default);

@@ -346,16 +346,18 @@ __device__ __forceinline__ TimeFactors eval_time_factors(double omega, double dt
 // Time factors of the step being computed, in the arithmetic type T. Three FP64 cosines per thread
 // took 6 of the 11.5 us of a 128 x 64 step (GB300 runs FP64 at a 64th of its FP32 rate), so
 // sequences of steps read them from a table that one small launch fills (launch_time_factors).
-template <class T>
+// EVAL = false: the caller always has the table (the cosine's slow path is a call with local memory,
+// which the warp-specialised kernels' register split does not go with).
+template <class T, bool EVAL>
 __device__ __forceinline__ void time_factors(const StepParams &p, T &ct, T &cth, T &cwh) {
     if (__double_as_longlong(p.omega) == 0) {  // (an FP64 comparison would cost more)
         ct = cth = sizeof(T) == 4 ? (T)p.fcoef[2] : (T)p.inv_c;
         cwh = T(1);
-    } else if (p.tfac) {
+    } else if (!EVAL || p.tfac) {
         const TimeFactors *f = p.tfac + p.step_off;
         if constexpr (sizeof(T) == 4) { ct = __ldg(&f->fct); cth = __ldg(&f->fcth); cwh = __ldg(&f->fcwh); }
         else { ct = __ldg(&f->ct); cth = __ldg(&f->cth); cwh = __ldg(&f->cwh); }
-    } else {
+    } else if constexpr (EVAL) {
         const TimeFactors f = eval_time_factors(p.omega, p.dt, p.inv_c, (double)(*p.step_ctr) + (double)p.step_off);
         ct = (T)f.ct;
         cth = (T)f.cth;
@@ -364,12 +366,21 @@ __device__ __forceinline__ void time_factors(const StepParams &p, T &ct, T &cth,
 }
 
 // Coefficients in the arithmetic type T.
+struct FromTable {};  // selects time_factors without the evaluation
 template <class T>
 struct Coef {
     T rho0, inv_rho0, inv_c, b1, c1, b7, c7, kappa, two_kappa, wcell, wface;
     T ct, cth;  // cos(omega t_n) / c and cos(omega (t_n + h)) / c: the time factors of G
     T cwh;      // cos(omega (t_n + h)): the time factor of an oscillating wall pressure
     __device__ __forceinline__ explicit Coef(const StepParams &p) {
+        coefficients(p);
+        time_factors<T, true>(p, ct, cth, cwh);
+    }
+    __device__ __forceinline__ Coef(const StepParams &p, FromTable) {
+        coefficients(p);
+        time_factors<T, false>(p, ct, cth, cwh);
+    }
+    __device__ __forceinline__ void coefficients(const StepParams &p) {
         if constexpr (sizeof(T) == 4) {  // rounded on the host (finish_step_params)
             rho0 = p.fcoef[0]; inv_rho0 = p.fcoef[1]; inv_c = p.fcoef[2]; b1 = p.fcoef[3]; c1 = p.fcoef[4];
             b7 = p.fcoef[5]; c7 = p.fcoef[6]; kappa = p.fcoef[7]; two_kappa = p.fcoef[8]; wcell = p.fcoef[9];
@@ -379,7 +390,6 @@ struct Coef {
             b7 = (T)p.b7; c7 = (T)p.c7; kappa = (T)p.kappa; two_kappa = (T)p.two_kappa; wcell = (T)p.wcell;
             wface = (T)p.wface;
         }
-        time_factors<T>(p, ct, cth, cwh);
     }
 };
 

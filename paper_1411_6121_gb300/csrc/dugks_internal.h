@@ -33,10 +33,10 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
 cudaError_t launch_step_q9(const StepParams &p, int store, int tx, int ty, cudaStream_t stream);
 cudaError_t launch_step_q19(const StepParams &p, int store, int tx, int ty, cudaStream_t stream);
 cudaError_t launch_step_q27(const StepParams &p, int store, int tx, int ty, cudaStream_t stream);
-// Throughput kernel for D3Q19 with F32/BF16/F16 storage (dugks_step3d.cuh); ry = CTA rows.
+// Throughput kernels for D3Q19 and D3Q27 with F32/BF16/F16 storage: ry 0 the warp-specialised one
+// (dugks_step3d_ws.cuh), else the non-specialised one (dugks_step3d.cuh) with ry CTA rows (D3Q27: 8).
 cudaError_t launch_step3d_q19(const StepParams &p, int store, int ry, cudaStream_t stream);
-// The same throughput kernel for D3Q27 (32 x 8 columns per CTA).
-cudaError_t launch_step3d_q27(const StepParams &p, int store, cudaStream_t stream);
+cudaError_t launch_step3d_q27(const StepParams &p, int store, int ry, cudaStream_t stream);
 // Throughput kernel for D2Q9 with F32/BF16/F16 storage (dugks_step2d.cuh; BF16:
 // dugks_step2d_cell.cuh): ry = block rows, tiles of step2d_tile_columns(store) columns x (ry - 2) rows (ry 0: chosen by the mesh; the results do not
 // depend on it). The batch form walks a work list of (instance, x0, y0) tile origins over
@@ -53,6 +53,7 @@ cudaError_t launch_step2d_batch_bf16(const StepParams *params, const int4 *items
 // Whether a TMA wait of the 3D throughput kernel gave up since the last call (the kernel then
 // skipped its step); clears the flag. 1: yes, 0: no, -1: the flag could not be read.
 int tma_wait_failures();
+int tma_wait_failures_q27();
 
 // Auxiliary kernels (aux.cu).
 cudaError_t launch_init(int q, int store, const StepParams &p, const double *pres, const double *vel, double rt,

@@ -1,11 +1,13 @@
-// step3d_q27.cu -- the throughput kernel of dugks_step3d.cuh instantiated for D3Q27 (the
-// paper's 3D velocity set, Sec. 2.3): 32 x 8 columns per CTA, F32/BF16/F16 storage. At
-// 27 velocities the TMA stages do not fit beside the ring, so every plane is loaded
-// directly (the kernel's tensor-map argument is unused).
+// step3d_q27.cu -- the 3D throughput kernels instantiated for D3Q27 (the paper's 3D velocity set,
+// Sec. 2.3), F32/BF16/F16 storage: the warp-specialised one (dugks_step3d_ws.cuh, the default) and
+// the non-specialised one (dugks_step3d.cuh, 32 x 8 columns per CTA; at 27 velocities its TMA
+// stages do not fit beside the ring, so every plane is loaded directly and the tensor map is
+// unused).
 #include <string.h>
 
 #include "dugks_internal.h"
 #include "dugks_step3d.cuh"
+#include "dugks_step3d_ws.cuh"
 
 namespace dugks {
 
@@ -48,12 +50,29 @@ static cudaError_t launch27(const StepParams &p, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_step3d_q27(const StepParams &p, int store, cudaStream_t stream) {
+// Whether a wait of this translation unit's kernels gave up since the last call (and clears it).
+int tma_wait_failures_q27() {
+    int v = 0;
+    if (cudaMemcpyFromSymbol(&v, g_tma_wait_failed, sizeof v) != cudaSuccess) return -1;
+    if (v) {
+        const int zero = 0;
+        cudaMemcpyToSymbol(g_tma_wait_failed, &zero, sizeof zero);
+    }
+    return v;
+}
+
+template <class S>
+static cudaError_t launch_s(const StepParams &p, int ry, cudaStream_t stream) {
     const bool force = p.field != nullptr || p.g[0] != 0.0 || p.g[1] != 0.0 || p.g[2] != 0.0;
+    if (ry == 0) return force ? launch_ws<27, S, true>(p, stream) : launch_ws<27, S, false>(p, stream);
+    return force ? launch27<S, true>(p, stream) : launch27<S, false>(p, stream);
+}
+
+cudaError_t launch_step3d_q27(const StepParams &p, int store, int ry, cudaStream_t stream) {
     switch (store) {
-        case 0: return force ? launch27<float, true>(p, stream) : launch27<float, false>(p, stream);
-        case 1: return force ? launch27<__nv_bfloat16, true>(p, stream) : launch27<__nv_bfloat16, false>(p, stream);
-        case 2: return force ? launch27<__half, true>(p, stream) : launch27<__half, false>(p, stream);
+        case 0: return launch_s<float>(p, ry, stream);
+        case 1: return launch_s<__nv_bfloat16>(p, ry, stream);
+        case 2: return launch_s<__half>(p, ry, stream);
     }
     return cudaErrorNotSupported;
 }

@@ -1,7 +1,7 @@
-"""The 2D step kernels at the edges of their tiles, element by element against the oracle: sizes one
+"""The step kernels at the edges of their tiles, element by element against the oracle: sizes one
 below, at and one above the columns and rows of a tile, odd sizes (the last column alone in its
 lane), every wall type on both axes, with and without a force; and the same bits whatever the
-block's rows."""
+block's rows (2D)."""
 import numpy as np
 import pytest
 
@@ -68,3 +68,20 @@ def test_d2q9_f16_one_step(shape):
     s.step(1)
     ref, got = _state(o), s.get_state().astype(np.float64) / 4096.0
     assert np.all(np.abs(got - ref) <= 2e-6 * np.abs(ref).max() + 2.0 ** -10 * np.abs(ref))
+
+
+FLOWS_3D = {
+    "channel": dict(bcs=W.channel_bcs(3), g=(1e-4, -2e-5, 3e-5), omega=0.2),
+    "cavity": dict(bcs=W.cavity_bcs(3, 0.1)),
+    "box": dict(bcs=[W.pressure(1e-3), W.bounce_back((0.0, 0.02, 0.0)), W.bounce_back(), W.wall((0.03, 0.0, 0.0)),
+                     W.wall(), W.bounce_back()], g=(0.0, 1e-4, 0.0)),
+}
+
+
+@pytest.mark.parametrize("q", [19, 27])
+@pytest.mark.parametrize("flow", sorted(FLOWS_3D))
+@pytest.mark.parametrize("shape", [(29, 5, 2), (30, 6, 9), (31, 7, 17), (61, 13, 3)])
+def test_3d_tile_edges(shape, flow, q):
+    cfg = dict(shape=shape, q=q, nu=0.05, dt=0.5, **FLOWS_3D[flow])
+    ref, got = _pair(cfg, 6)
+    assert np.abs(got - ref).max() < 2e-6 * np.abs(ref).max()
