@@ -83,8 +83,8 @@ typedef struct {
     int64_t nz;      /* 1 in 2D */
     double dx;       /* uniform spacing, dx = dy = dz */
     const double *faces[3]; /* optional non-uniform mesh (Sec. 3.4's tanh mesh, which
-                               Sec. 3.5 also uses for the cube; 2D and 3D, the reference
-                               kernel, no adjoint or batch): HOST arrays of the n+1
+                               Sec. 3.5 also uses for the cube; 2D and 3D, no adjoint
+                               or batch; 3D: the reference kernel): HOST arrays of the n+1
                                interface coordinates of x, y (and z in 3D), copied at
                                creation; NULL (default) means uniform spacing dx along that
                                axis. F32 or F64 storage; 16-bit storage: the handle is not

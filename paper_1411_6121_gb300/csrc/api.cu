@@ -98,6 +98,7 @@ StepParams dugks::handle_params(const dugks_t h) {
 }
 
 cudaError_t dugks::handle_launch_step(dugks_t h, StepParams &p) {
+    if (h->lean) return launch_step2d_lean(p, h->store, h->stream);
     if (h->kernel == 0 && h->q == 19 && h->store != DUGKS_STORE_F64)
         return launch_step3d_q19(p, h->store, h->ry3d, h->stream);
     if (h->kernel == 0 && h->q == 27 && h->store != DUGKS_STORE_F64) return launch_step3d_q27(p, h->store, h->ry3d, h->stream);
@@ -192,6 +193,10 @@ int dugks_create(const dugks_mesh *mesh, int32_t lattice, double nu, double dt, 
         return handle_fail(NULL, DUGKS_E_INVAL, "a 2D mesh has no z interface coordinates");
     const bool nonuni = mesh->faces[0] || mesh->faces[1] || (dim == 3 && mesh->faces[2]);
     double hmin = mesh->dx;  // smallest cell width (CFL)
+    // 2D FP64 and non-uniform meshes by default: the kernel with few operations per cell (a quarter of
+    // the reference kernel's FP64 instructions); a tile or kernel asked for takes the reference one
+    const bool lean = dim == 2 && o.model == DUGKS_MODEL_INCOMPRESSIBLE && o.kernel == 0 && o.tile_x == 0 && o.tile_y == 0 &&
+                      (o.store == DUGKS_STORE_F64 || (nonuni && o.store == DUGKS_STORE_F32));
     if (nonuni) {
         hmin = INFINITY;
         for (int a = 0; a < dim; a++)
@@ -280,6 +285,7 @@ int dugks_create(const dugks_mesh *mesh, int32_t lattice, double nu, double dt, 
     h->tile_y = ty;
     h->kernel = o.kernel;
     h->model = o.model;
+    h->lean = lean;
     h->ry3d = ry3d;
     h->esize = o.store == DUGKS_STORE_F32 ? 4 : (o.store == DUGKS_STORE_F64 ? 8 : 2);
     h->state_bytes = (size_t)h->q * h->px * h->ny * h->nz * h->esize;

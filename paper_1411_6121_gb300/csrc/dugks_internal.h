@@ -50,6 +50,10 @@ cudaError_t launch_step2d_q9_bf16(const StepParams &p, int ry, cudaStream_t stre
 cudaError_t launch_step2d_batch_bf16(const StepParams *params, const int4 *items, int nitems, int parity, int ry,
                                      bool force, cudaStream_t stream);
 
+// D2Q9 kernel with few operations per cell (dugks_step2d_lean.cuh): F64 storage, and non-uniform meshes
+// with F32 or F64 storage; incompressible model.
+cudaError_t launch_step2d_lean(const StepParams &p, int store, cudaStream_t stream);
+
 // Whether a TMA wait of the 3D throughput kernel gave up since the last call (the kernel then
 // skipped its step); clears the flag. 1: yes, 0: no, -1: the flag could not be read.
 int tma_wait_failures();

@@ -54,6 +54,7 @@ struct dugks_s {
     int use_graph, tile_x, tile_y;
     int kernel;            // 0: throughput kernel where built, 1: reference kernel
     int model;             // DUGKS_MODEL_*
+    bool lean;             // 2D: the kernel with few operations (FP64, non-uniform meshes)
     double *d_metric;      // non-uniform mesh metrics (device; NULL: uniform), see StepParams
     double eg[3][2];       // its ghost extrapolation coefficients
     int64_t metric_off[3]; // offset of each axis' block in d_metric

@@ -85,3 +85,34 @@ def test_3d_tile_edges(shape, flow, q):
     cfg = dict(shape=shape, q=q, nu=0.05, dt=0.5, **FLOWS_3D[flow])
     ref, got = _pair(cfg, 6)
     assert np.abs(got - ref).max() < 2e-6 * np.abs(ref).max()
+
+
+# The kernel of FP64 storage and of non-uniform meshes: tiles of 30 columns and up to 6 rows. The
+# tolerances are those of a step's rounding in either type (as in the parity tests), for 10 steps.
+@pytest.mark.parametrize("flow", sorted(FLOWS))
+@pytest.mark.parametrize("shape", [(2, 2), (29, 7), (30, 6), (31, 13), (61, 5)])
+@pytest.mark.parametrize("mesh,store", [("uniform", 3), ("tanh", 3), ("tanh", 0)])
+def test_d2q9_lean_tile_edges(mesh, store, shape, flow):
+    cfg = dict(shape=shape, q=9, nu=0.05, dt=0.5, **FLOWS[flow])
+    if mesh == "tanh":
+        faces = [W.tanh_faces(n, n) for n in shape]
+        cfg.update(faces=faces, dt=0.5 * min(np.diff(f).min() for f in faces))
+    ref, got = _pair(cfg, 10, store=store)
+    assert np.abs(got - ref).max() < (1e-11 if store == 3 else 2e-6) * np.abs(ref).max()
+
+
+def test_d2q9_lean_matches_reference_kernel_with_field():
+    """The default route of FP64 against the general kernel (kernel=1): a field, an oscillating
+    acceleration, both orders of the walls."""
+    import torch
+    from paper_1411_6121_gb300 import dugks
+    shape = (43, 19)
+    fld = torch.tensor(W.force_field(shape, 2e-5, seed=2, rel=0.5), dtype=torch.float32, device="cuda")
+    for bcs in (W.channel_bcs(2), W.channel_bcs(2)[2:] + W.channel_bcs(2)[:2]):
+        outs = []
+        for kernel in (0, 1):
+            s = dugks.Sim(shape, q=9, nu=0.05, dt=0.5, g=(1e-5, 2e-5, 0.0), omega=0.3, bcs=bcs, field=fld, store=3, kernel=kernel)
+            s.init(*W.random_state_fields(shape, seed=4, u_amp=0.03, p_amp=1e-3))
+            s.step(10)
+            outs.append(s.get_state())
+        assert np.abs(outs[0] - outs[1]).max() < 1e-11 * np.abs(outs[1]).max()
