@@ -31,8 +31,8 @@
 //  * At a wall interface step 5 replaces the incoming velocities' F: the interface moments get
 //    the sum of the changes, and the cell's La the changes themselves.
 // Measured (us per step, one instance, before / now; before: one cell per thread, 32 x 8 threads, 30
-// warp instructions per cell, 56% issue): 1024^2 cavity 40.0 / 27.2 (18 instructions per cell, 53%
-// issue, 24 warps per SM), 2048^2 155 / 102, 512 x 256 channel 8.8 / 6.8, 8 x 32 channel 3.45 / 3.4 (the
+// warp instructions per cell, 56% issue): 1024^2 cavity 40.0 / 27.2 (16 instructions per cell, 53%
+// issue, 24 warps per SM), 2048^2 155 / 102, 512 x 256 channel 8.8 / 6.8, 8 x 32 channel 3.45 / 3.2 (the
 // latency of one block).
 #pragma once
 
@@ -219,13 +219,18 @@ __device__ __forceinline__ void make_row(const StepParams &p, const Coef<float> 
     if constexpr (FORCE) gm = mul(fma(G[0], m[0], mul(G[1], m[1])), bc(cf.inv_rho0));
     const V base = fma(bc(-1.5f * cf.inv_rho0), mm, drho), c45 = bc(4.5f * cf.inv_rho0);
     const V b1 = bc(cf.b1), b43 = bc(cf.b1 * (4.0f / 3.0f)), t43 = bc(4.0f / 3.0f);
+    // The weights are 1/9 times 4, 1 and 1/4, so the axes' weight and its split serve all, with e.m and
+    // q of the diagonals a quarter and of the rest velocity four times (exact): four constants in
+    // registers instead of ten.
+    constexpr double W = 1.0 / 9.0;
+    constexpr float wh = (float)W, wl = (float)(W - (double)wh);
+    constexpr float w3h = (float)(3.0 * W), w3l = (float)(3.0 * W - (double)w3h);
+    const V qt = bc(0.25f), mq[2] = {mul(qt, m[0]), mul(qt, m[1])}, base4 = mul(qt, base), c45d = bc(18.0f * cf.inv_rho0);
     sfor<4>([&](auto jc) {
         constexpr int k = 5 + jc;  // (0, 1), (1, -1), (1, 0), (1, 1) and the opposite of each
-        constexpr double W = Lat<9>::wt<double>(k);
-        constexpr float wh = (float)W, wl = (float)(W - (double)wh);
-        constexpr float w3h = (float)(3.0 * W), w3l = (float)(3.0 * W - (double)w3h);
-        const V em = ex(k) == 0 ? m[1] : (ey(k) == 0 ? m[0] : (ey(k) > 0 ? add(m[0], m[1]) : sub(m[0], m[1])));
-        const V q = fma(mul(c45, em), em, base);
+        constexpr bool diag = ex(k) != 0 && ey(k) != 0;
+        const V em = diag ? (ey(k) > 0 ? add(mq[0], mq[1]) : sub(mq[0], mq[1])) : (ex(k) == 0 ? m[1] : m[0]);
+        const V q = diag ? fma(mul(c45d, em), em, base4) : fma(mul(c45, em), em, base);
         const V wq = fma(bc(wl), q, mul(bc(wh), q));
         const V en = sub(bc(0.0f), em);
         const V gp = fma(bc(w3h), em, fma(bc(w3l), em, wq)), gn = fma(bc(w3h), en, fma(bc(w3l), en, wq));
@@ -237,7 +242,8 @@ __device__ __forceinline__ void make_row(const StepParams &p, const Coef<float> 
             u0[8 - k] = fma(b43, dn, g[8 - k]);
         } else {
             const V ge = ex(k) == 0 ? G[1] : (ey(k) == 0 ? G[0] : (ey(k) > 0 ? add(G[0], G[1]) : sub(G[0], G[1])));
-            const V fqp = fma(bc((float)W), bc(cf.rho0), gp), fqn = fma(bc((float)W), bc(cf.rho0), gn);
+            const V r0 = bc(diag ? 0.25f * cf.rho0 : cf.rho0);
+            const V fqp = fma(bc(wh), r0, gp), fqn = fma(bc(wh), r0, gn);
             const V c3 = bc(3.0f * cf.c1), n3 = bc(-3.0f * cf.c1);
             const V ip = fma(mul(c3, sub(ge, gm)), fqp, mul(b1, dp)), in = fma(mul(n3, add(ge, gm)), fqn, mul(b1, dn));
             r.f[k] = add(g[k], ip);
@@ -247,11 +253,9 @@ __device__ __forceinline__ void make_row(const StepParams &p, const Coef<float> 
         }
     });
     {
-        constexpr double W = Lat<9>::wt<double>(4);
-        constexpr float wh = (float)W, wl = (float)(W - (double)wh);
-        const V gq = fma(bc(wl), base, mul(bc(wh), base));
+        const V b4 = mul(bc(4.0f), base), gq = fma(bc(wl), b4, mul(bc(wh), b4));
         V in = mul(b1, sub(gq, g[4]));
-        if constexpr (FORCE) in = fma(mul(bc(-3.0f * cf.c1), gm), fma(bc((float)W), bc(cf.rho0), gq), in);
+        if constexpr (FORCE) in = fma(mul(bc(-3.0f * cf.c1), gm), fma(bc(wh), bc(4.0f * cf.rho0), gq), in);
         r.f[4] = add(g[4], in);
         u0[4] = fma(t43, in, g[4]);
     }

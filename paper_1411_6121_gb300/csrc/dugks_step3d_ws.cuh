@@ -45,8 +45,8 @@
 // flag, then the group leaves together; see tma.cuh).
 // Measured (256^3 cavity unless stated, FP32, ms per step before / now; D3Q19 before: step-4 values formed
 // at every interface by this kernel's first form, D3Q27 before: the non-specialised kernel): D3Q19
-// 1.492 / 1.369, with a force 1.927 / 1.630, BF16 1.556 / 1.435; D3Q27 3.81 / 2.82, forced 157 x 101 x 83
-// 0.545 / 0.368. At 128^3 63 warp instructions per cell, 52% issue.
+// 1.492 / 1.324, with a force 1.927 / 1.608, BF16 1.556 / 1.380; D3Q27 3.81 / 2.62, forced 157 x 101 x 83
+// 0.545 / 0.367. At 128^3 62 warp instructions per cell, 53% issue.
 #pragma once
 
 #include <math.h>
@@ -128,9 +128,13 @@ struct ShapeWS {
     static constexpr int NSLOT = 4, NU0 = U0 ? 3 : 0;
     static constexpr int NUC = TYI * RX;              // columns that update (rows 1 .. TYI)
     static constexpr int PLANE = RY * RX * CS;
-    // ring; B_y of rows 1..RY-1; numbers at +y of rows 0..RY-2; wall terms of the low and high y wall;
-    // u0 pairs and rest of rows 1..TYI
-    static constexpr int XB = (RY - 1) * RX * 4, YV = (RY - 1) * RX * NV, WT = 2 * RX * 2 * P::NX;
+    // Without a force every row forms the numbers of both its y interfaces from the parts A_y, B_y of
+    // its neighbours (double-buffered, one barrier per plane); with one, where they are many, each
+    // interface's are formed once and published behind a second barrier.
+    static constexpr bool BOTH_Y = !FORCE;
+    // ring; A_y and B_y of all rows; numbers at +y of rows 0..RY-2; wall terms of the low and high y
+    // wall; u0 pairs and rest of rows 1..TYI
+    static constexpr int XB = (BOTH_Y ? 2 : 1) * RY * RX * 8, YV = BOTH_Y ? 0 : (RY - 1) * RX * NV, WT = 2 * 2 * RX * 2 * P::NX;
     static constexpr size_t FLOATS = (size_t)NSLOT * PLANE + XB + YV + WT + (size_t)NU0 * NUC * (UP + 1);
     static_assert(PLANE % 4 == 0 && XB % 4 == 0 && YV % 4 == 0 && WT % 4 == 0, "vector accesses must stay aligned");
     static constexpr int BX = 32 + (sizeof(S) == 4 ? 4 : 8);  // TMA box width (start rounded down)
@@ -226,8 +230,8 @@ __device__ __forceinline__ void step1_pairs(const float2 *G, float g9, const flo
         constexpr float wh = (float)W, wl = (float)(W - (double)wh);
         constexpr float w3h = (float)(3.0 * W), w3l = (float)(3.0 * W - (double)w3h);
         const float wq = fmaf(wl, q, wh * q);
-        const float2 EM = f2(em, em);
-        const float2 GEQ = __ffma2_rn(f2(w3h, -w3h), EM, __ffma2_rn(f2(w3l, -w3l), EM, f2(wq, wq)));
+        // scalar: the weights are immediates there, a packed operation would need them in registers
+        const float2 GEQ = f2(fmaf(w3h, em, fmaf(w3l, em, wq)), fmaf(-w3h, em, fmaf(-w3l, em, wq)));
         float2 F;
         const float2 D = sub2(GEQ, G[j]);
         if constexpr (FORCE) {
@@ -456,9 +460,9 @@ __global__ void __launch_bounds__(512, 1)
     const int x0 = blockIdx.x * K::TXI, y0 = blockIdx.y * K::TYI;
 
     float *ring = reinterpret_cast<float *>(smem_raw);  // [NSLOT][RY][32][CS]
-    float *xb = ring + K::NSLOT * K::PLANE;            // [rows 1..RY-1][32][4]: B_y
+    float *xb = ring + K::NSLOT * K::PLANE;            // [2][RY][32][8]: A_y, B_y (by the plane's parity)
     float *yv = xb + K::XB;                            // [rows 0..RY-2][NV][32]: numbers at +y
-    float *wt = yv + K::YV;                            // [2][32][2 NX]: terms of the low / high y wall
+    float *wt = yv + K::YV;                            // [2][2][32][2 NX]: terms of the low / high y wall
     float *u0b = wt + K::WT;                           // [NU0][rows 1..TYI][32][UP]
     float *u0r = u0b + K::NU0 * K::NUC * K::UP;        // [NU0][rows 1..TYI][32]: rest velocity
     unsigned char *stage = reinterpret_cast<unsigned char *>(
@@ -862,7 +866,7 @@ __global__ void __launch_bounds__(512, 1)
             if (lane >= 1 && lane <= K::TXI && gx < nx) {
                 float2 T[NX];
                 wall_term<Q, FORCE, 1>(p, ctx, ywlo ? row : row - 1, kz, ywlo ? 0 : ny, T);
-                float *o = wt + ((ywlo ? 0 : 1) * 32 + lane) * 2 * NX;
+                float *o = wt + (((kz & 1) * 2 + (ywlo ? 0 : 1)) * 32 + lane) * 2 * NX;
 #pragma unroll
                 for (int i = 0; i < NX; i++) st2(o + 2 * i, T[i]);
             }
@@ -877,13 +881,18 @@ __global__ void __launch_bounds__(512, 1)
             });
         }
         // ---- y parts of plane kz: publish B_y ----
-        float dz[4], Ay[4];
+        float dz[4], Ay[4], By[4];
+        float *xp = xb + ((K::BOTH_Y ? (kz & 1) * RY * 32 : 0) + row * 32 + lane) * 8;
         mdiff(prv, nxt, AZ, dz);
         if (ycol) {
             float B[4];
             mparts(AY, SA, cur, Mx, dz, Ay);
             mparts(AY, SB, cur, Mx, dz, B);
-            if (row >= 1) *reinterpret_cast<float4 *>(xb + ((row - 1) * 32 + lane) * 4) = make_float4(B[0], B[1], B[2], B[3]);
+            float4 *o = reinterpret_cast<float4 *>(xp);
+            if (K::BOTH_Y) o[0] = make_float4(Ay[0], Ay[1], Ay[2], Ay[3]);
+            o[1] = make_float4(B[0], B[1], B[2], B[3]);
+#pragma unroll
+            for (int i = 0; i < 4; i++) By[i] = B[i];
         }
         // ---- differences of the interfaces' numbers, or (FORCE) N: x by shuffles, z carried ----
         float DX[NV], DZ[NV];
@@ -969,32 +978,50 @@ __global__ void __launch_bounds__(512, 1)
                         La[j] = f2(fmaf(g, T.x, La[j].x), fmaf(-g, T.y, La[j].y));
                     });
                 };
-                if (gy == 0) wall(wt + lane * 2 * NX, -1.0f);
-                if (gy == ny - 1) wall(wt + (32 + lane) * 2 * NX, 1.0f);
+                const float *w = wt + ((kz & 1) * 64 + lane) * 2 * NX;
+                if (gy == 0) wall(w, -1.0f);
+                if (gy == ny - 1) wall(w + 64 * NX, 1.0f);
             }
         }
         float DY[NV];
-        if (need_y) {
-            if (ynwall) {
+        if constexpr (K::BOTH_Y) {
+            if (upd) {
+                const float G0[3] = {0.0f, 0.0f, 0.0f};
+                const float4 hb = *reinterpret_cast<const float4 *>(xp + 32 * 8 + 4), la = *reinterpret_cast<const float4 *>(xp - 32 * 8);
+                float V[NV];
+                const float fn4[4] = {Ay[0] + hb.x, Ay[1] + hb.y, Ay[2] + hb.z, Ay[3] + hb.w};
+                const float fs4[4] = {la.x + By[0], la.y + By[1], la.z + By[2], la.w + By[3]};
+                numbers(AY, fn4, G0, DY);
+                numbers(AY, fs4, G0, V);
+                const bool wn = !pery && gy == ny - 1, ws = !pery && gy == 0;  // warp-uniform
 #pragma unroll
-                for (int i = 0; i < NV; i++) DY[i] = 0.0f;
-            } else {
-                const float4 nb = *reinterpret_cast<const float4 *>(xb + (row * 32 + lane) * 4);  // row + 1's entry
-                const float fm[4] = {Ay[0] + nb.x, Ay[1] + nb.y, Ay[2] + nb.z, Ay[3] + nb.w};
-                float Gb[3], fy[3];
-                cell_field(gy + 1, kz, fy);
-                mean_G(fc, fy, Gb);
-                numbers(AY, fm, Gb, DY);
+                for (int i = 0; i < NV; i++) DY[i] = (wn ? 0.0f : DY[i]) - (ws ? 0.0f : V[i]);
             }
+        } else {
+            if (need_y) {
+                if (ynwall) {
 #pragma unroll
-            for (int i = 0; i < NV; i++) yv[(row * NV + i) * 32 + lane] = DY[i];
+                    for (int i = 0; i < NV; i++) DY[i] = 0.0f;
+                } else {
+                    const float4 nb = *reinterpret_cast<const float4 *>(xp + 32 * 8 + 4);  // row + 1's B
+                    const float fm[4] = {Ay[0] + nb.x, Ay[1] + nb.y, Ay[2] + nb.z, Ay[3] + nb.w};
+                    float Gb[3], fy[3];
+                    cell_field(gy + 1, kz, fy);
+                    mean_G(fc, fy, Gb);
+                    numbers(AY, fm, Gb, DY);
+                }
+#pragma unroll
+                for (int i = 0; i < NV; i++) yv[(row * NV + i) * 32 + lane] = DY[i];
+            }
+            cons_bar();
         }
-        cons_bar();
 
         // ---- steps 8-9, update of cell (gx, gy, kz) ----
         if (upd) {
+            if constexpr (!K::BOTH_Y) {
 #pragma unroll
-            for (int i = 0; i < NV; i++) DY[i] -= yv[((row - 1) * NV + i) * 32 + lane];
+                for (int i = 0; i < NV; i++) DY[i] -= yv[((row - 1) * NV + i) * 32 + lane];
+            }
             if constexpr (FORCE) add_N(AY, DY);
             // sums that the pairs of a coordinate plane, and the corners, share
             float o1[3], o2[3], e1[3], e2[3];  // planes xy, xz, yz
