@@ -2,9 +2,9 @@
 //
 // Every instance keeps its own mesh, viscosity, acceleration and boundaries; they share the
 // time step, RT, rho0 and the storage type. One time step of the whole batch is one
-// persistent launch (fused_step_batch) that walks a work list of (instance, tile) items,
-// largest instances first; dugks_batch_step replays n such launches as a captured CUDA
-// graph. The tile body is that of the D2Q9 throughput kernel (dugks_step2d.cuh) or of the
+// launch over a work list of (instance, tile) items, largest instances first: a block per item
+// (throughput tiles) or persistent blocks that walk the list (reference tiles);
+// dugks_batch_step replays n such launches as a captured CUDA graph. The tile body is that of the D2Q9 throughput kernel (dugks_step2d.cuh) or of the
 // reference kernel (dugks_step.cuh); the tile comes from a timing autotuner
 // (dugks_batch_tune) whose choice is cached per (instance sizes, storage, SM count).
 #include <math.h>

@@ -1,5 +1,5 @@
 // step2d_q9.cu -- instantiations and launchers of the D2Q9 throughput kernel
-// (dugks_step2d.cuh): one instance on a grid of tiles, or a batch on a persistent grid.
+// (dugks_step2d.cuh): one instance on a grid of tiles, or a batch on a list of them.
 #include <algorithm>
 
 #include "dugks_internal.h"
@@ -78,10 +78,9 @@ cudaError_t launch_many(const StepParams *params, const int4 *items, int nitems,
     const Residency *r;
     cudaError_t e = configure<S, FORCE, true>(&r);
     if (e != cudaSuccess) return e;
-    const int grid = std::min(nitems, r->sms * r->blocks[ry]);  // persistent: the resident blocks, at most the items
-    if (grid < 1) return cudaSuccess;
-    return launch_chained(fused_step2d_batch<S, FORCE>, dim3(grid), dim3(32, ry), m2::smem_bytes<FORCE != 0>(ry), stream,
-                          params, items, nitems, parity);
+    if (nitems < 1) return cudaSuccess;
+    return launch_chained(fused_step2d_batch<S, FORCE>, dim3(nitems), dim3(32, ry), m2::smem_bytes<FORCE != 0>(ry), stream,
+                          params, items, parity);
 }
 
 template <class S>
