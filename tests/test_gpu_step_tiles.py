@@ -116,3 +116,20 @@ def test_d2q9_lean_matches_reference_kernel_with_field():
             s.step(10)
             outs.append(s.get_state())
         assert np.abs(outs[0] - outs[1]).max() < 1e-11 * np.abs(outs[1]).max()
+
+
+@pytest.mark.parametrize("shapes", [[(2, 2), (300, 171)], [(511, 257), (7, 5)]])
+def test_batch_read_back_by_pieces(shapes):
+    """Moments read to the host by page-locked pieces: instances below, and of several (odd) pieces;
+    the same values as the moments of the single instance."""
+    from paper_1411_6121_gb300 import dugks
+    ins = [dict(shape=s, nu=0.05, bcs=W.cavity_bcs(2, 0.1)) for s in shapes]
+    b = dugks.Batch(ins, dt=0.5)
+    for i, s in enumerate(shapes):
+        p, u = W.random_state_fields(s, seed=7, u_amp=0.03, p_amp=1e-3)
+        b.init(i, p=p, u=u)
+        one = dugks.Sim(q=9, dt=0.5, tile=(32, 8), kernel=0, **ins[i])
+        one.init(p=p, u=u)
+        assert np.array_equal(b.moments(i), one.moments())
+        one.close()
+    b.close()
