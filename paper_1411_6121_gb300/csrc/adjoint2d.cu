@@ -94,105 +94,24 @@ __device__ __forceinline__ int64_t fidx(const AdjParams<T> &a, int d, int i, int
 }
 
 // ---- step 2: extended positions -1 .. n along one axis (reading R3: ghost = 2 f(0) - f(1)
-// at a wall, the periodic image otherwise) ----
-// The transpose: positions that cell x contributes to and the weights (at most 3).
-template <class T>
-__device__ __forceinline__ int ext_users(int x, int n, int per, int c[3], T w[3]) {
-    int k = 0;
-    c[k] = x; w[k++] = T(1);
-    if (per) {
-        if (x == n - 1) { c[k] = -1; w[k++] = T(1); }
-        if (x == 0) { c[k] = n; w[k++] = T(1); }
-    } else {
-        if (x == 0) { c[k] = -1; w[k++] = T(2); }
-        if (x == 1) { c[k] = -1; w[k++] = T(-1); }
-        if (x == n - 1) { c[k] = n; w[k++] = T(2); }
-        if (x == n - 2) { c[k] = n; w[k++] = T(-1); }
-    }
-    return k;
-}
-
-// fbar+ at an extended position, branch-free: always two cells per axis (the second with
-// weight 0 where the position is a real cell or a periodic image), so every load address is
-// known up front and the loads of a reconstruction can all be in flight together.
+// at a wall, the periodic image otherwise), as two cells and their weights (the second 0 where the
+// position is a real cell or an image): branch-free, so the loads of an item are all in flight
+// together ----
 template <class T>
 __device__ __forceinline__ void ext2(int x, int n, int per, int c[2], T w[2]) {
-    if (x >= 0 && x < n) { c[0] = x; c[1] = x; w[0] = T(1); w[1] = T(0); }
-    else if (per) { c[0] = x < 0 ? x + n : x - n; c[1] = c[0]; w[0] = T(1); w[1] = T(0); }
-    else { c[0] = x < 0 ? 0 : n - 1; c[1] = x < 0 ? 1 : n - 2; w[0] = T(2); w[1] = T(-1); }
-}
-template <class T>
-__device__ __forceinline__ T phi_ext(const AdjParams<T> &a, int k, int x, int y) {
-    int cx[2], cy[2];
-    T wx[2], wy[2];
-    ext2<T>(x, a.n[0], a.per[0], cx, wx);
-    ext2<T>(y, a.n[1], a.per[1], cy, wy);
-    const T *ph = a.phi + k * ncell(a);
-    const int64_t r0 = (int64_t)a.n[0] * cy[0], r1 = (int64_t)a.n[0] * cy[1];
-    const T p00 = ph[cx[0] + r0], p10 = ph[cx[1] + r0], p01 = ph[cx[0] + r1], p11 = ph[cx[1] + r1];
-    return wy[0] * (wx[0] * p00 + wx[1] * p10) + wy[1] * (wx[0] * p01 + wx[1] * p11);
+    const bool lo = x < 0, out = lo || x >= n, wall = out && !per;
+    c[0] = wall ? (lo ? 0 : n - 1) : (out ? (lo ? n - 1 : 0) : x);
+    c[1] = wall ? (lo ? 1 : n - 2) : c[0];
+    w[0] = wall ? T(2) : T(1);
+    w[1] = wall ? T(-1) : T(0);
 }
 
-// ---- steps 3-4: step-4 value of velocity k at interface (d, i, j) (eq. (23) with the
-// step-3 cross points): 1/2 (L + R) - kappa e_d (R - L) - kappa/4 e_t [(L+R)_{t+1} - (L+R)_{t-1}] ----
-template <class T>
-__device__ __forceinline__ T recon(const AdjParams<T> &a, int d, int i, int j, int k) {
-    const int ed = L9::e(k, d), et = L9::e(k, 1 - d);
-    const int lx = d == 0 ? i - 1 : i, ly = d == 1 ? j - 1 : j;
-    const T l = phi_ext(a, k, lx, ly), r = phi_ext(a, k, i, j);
-    T v = T(0.5) * (l + r) - a.kappa * (T)ed * (r - l);
-    if (et) {
-        const int tx = d == 0 ? 0 : 1, ty = d == 0 ? 1 : 0;
-        const T pp = phi_ext(a, k, lx + tx, ly + ty) + phi_ext(a, k, i + tx, j + ty);
-        const T pm = phi_ext(a, k, lx - tx, ly - ty) + phi_ext(a, k, i - tx, j - ty);
-        v -= T(0.25) * a.kappa * (T)et * (pp - pm);
-    }
-    return v;
-}
-
-// Transpose of recon: d/d fbar+(x, y) of sum over interfaces of fb . F (velocity k).
-template <class T>
-__device__ __forceinline__ T recon_T(const AdjParams<T> &a, int k, int x, int y) {
-    const int ex = L9::e(k, 0), ey = L9::e(k, 1);
-    const int64_t n0 = nface(a, 0), n1 = nface(a, 1);
-    const T *f0 = a.fb[0] + k * n0, *f1 = a.fb[1] + k * n1;
-    // branch-free: the index is clamped into range and the value masked, so the loads do
-    // not wait on one another
-    auto fx = [&](int i, int j) -> T {
-        const bool in = !(i < 0 || i > a.n[0] || j < 0 || j >= a.n[1]);
-        const T v = f0[fidx(a, 0, min(max(i, 0), a.n[0]), min(max(j, 0), a.n[1] - 1))];
-        return in ? v : T(0);
-    };
-    auto fy = [&](int i, int j) -> T {
-        const bool in = !(i < 0 || i >= a.n[0] || j < 0 || j > a.n[1]);
-        const T v = f1[fidx(a, 1, min(max(i, 0), a.n[0] - 1), min(max(j, 0), a.n[1]))];
-        return in ? v : T(0);
-    };
-    const T h = T(0.5), q = T(0.25) * a.kappa;
-    // as L of x interface (x+1, y), R of (x, y); as a tangential neighbour of the x
-    // interfaces of rows y-1 (their t+1 pair) and y+1 (their t-1 pair)
-    T v = (h + a.kappa * ex) * fx(x + 1, y) + (h - a.kappa * ex) * fx(x, y);
-    if (ey) v += q * (T)ey * ((fx(x + 1, y + 1) + fx(x, y + 1)) - (fx(x + 1, y - 1) + fx(x, y - 1)));
-    // the same for the y interfaces, tangential along x
-    v += (h + a.kappa * ey) * fy(x, y + 1) + (h - a.kappa * ey) * fy(x, y);
-    if (ex) v += q * (T)ex * ((fy(x + 1, y + 1) + fy(x + 1, y)) - (fy(x - 1, y + 1) + fy(x - 1, y)));
-    return v;
-}
-
-// ---- equilibrium (eq. (6), deviation form, m = rho0 u / c) and its derivative ----
+// ---- equilibrium (eq. (6), deviation form, m = rho0 u / c) ----
 template <class T>
 __device__ __forceinline__ T geq(const AdjParams<T> &a, int k, T dr, const T m[2]) {
     const T em = (T)L9::e(k, 0) * m[0] + (T)L9::e(k, 1) * m[1];
     const T mm = m[0] * m[0] + m[1] * m[1];
     return L9::wt<T>(k) * (dr + T(3) * em + (T(4.5) * em * em - T(1.5) * mm) * a.inv_rho0);
-}
-template <class T>
-__device__ __forceinline__ void geq_dm(const AdjParams<T> &a, int k, const T m[2], T out[2]) {
-    const T e0 = (T)L9::e(k, 0), e1 = (T)L9::e(k, 1);
-    const T em = e0 * m[0] + e1 * m[1];
-    const T W = L9::wt<T>(k);
-    out[0] = W * (T(3) * e0 + (T(9) * em * e0 - T(3) * m[0]) * a.inv_rho0);
-    out[1] = W * (T(3) * e1 + (T(9) * em * e1 - T(3) * m[1]) * a.inv_rho0);
 }
 
 // Moments of a distribution with the force weight w (dt/2 at cells, h/2 at interfaces).
@@ -223,26 +142,54 @@ __device__ __forceinline__ T wsum(T v) {
     return v;
 }
 
-// Relaxation P_k = f_k + b (geq_k - f_k) + c S_k with S_k = 3 (Gh.e_k - Gh.m/rho0) f_eq,k
-// (steps 1 and 7). Given the weight w = dL/dP_k of one velocity k, its share of dL/d(drho),
-// dL/dm and dL/dGh through the moment dependence (the direct part (1 - b) w is left to the
-// caller); summed over the velocities by the caller.
+// The lane's velocity: k < Q, lanes beyond it repeat velocity 0 and take part with zeros.
 template <class T>
-__device__ __forceinline__ void relax_T_one(const AdjParams<T> &a, int k, T w, T dr, const T m[2], const T Gh[2],
-                                            T b, T c, T &bdr, T bm[2], T bG[2]) {
+struct LaneVel {
+    int k, ie[2];
+    bool act;
+    T e[2], W;
+    __device__ __forceinline__ LaneVel() {
+        const int lane = half_lane();
+        act = lane < Q;
+        k = act ? lane : 0;
+        ie[0] = k / 3 - 1;
+        ie[1] = k - 3 * (k / 3) - 1;
+        e[0] = (T)ie[0];
+        e[1] = (T)ie[1];
+        W = ie[0] && ie[1] ? T(1) / T(36) : (ie[0] || ie[1] ? T(1) / T(9) : T(4) / T(9));
+    }
+};
+template <class T>
+__device__ __forceinline__ T geq_lane(const LaneVel<T> &l, T inv_rho0, T dr, const T m[2]) {
+    const T em = l.e[0] * m[0] + l.e[1] * m[1], mm = m[0] * m[0] + m[1] * m[1];
+    return l.W * (dr + T(3) * em + (T(4.5) * em * em - T(1.5) * mm) * inv_rho0);
+}
+template <class T>
+__device__ __forceinline__ void geq_dm_lane(const LaneVel<T> &l, T inv_rho0, const T m[2], T out[2]) {
+    const T em9 = T(9) * (l.e[0] * m[0] + l.e[1] * m[1]);
+#pragma unroll
+    for (int c = 0; c < 2; c++) out[c] = l.W * (T(3) * l.e[c] + (em9 * l.e[c] - T(3) * m[c]) * inv_rho0);
+}
+
+// Relaxation P_k = f_k + b (geq_k - f_k) + c S_k with S_k = 3 (Gh.e_k - Gh.m/rho0) f_eq,k
+// (steps 1 and 7). Given the weight w = dL/dP_k of the lane's velocity, dL/d(drho), dL/dm and dL/dGh
+// through the moment dependence (the direct part (1 - b) w is left to the caller), summed over
+// the velocities.
+template <class T>
+__device__ __forceinline__ void relax_T_lane(const AdjParams<T> &a, const LaneVel<T> &l, T w, T dr, const T m[2],
+                                             const T Gh[2], T b, T c, T &bdr, T bm[2], T bG[2]) {
     const T gm = (Gh[0] * m[0] + Gh[1] * m[1]) * a.inv_rho0;
-    const T e0 = (T)L9::e(k, 0), e1 = (T)L9::e(k, 1);
-    const T W = L9::wt<T>(k);
-    const T s = T(3) * (Gh[0] * e0 + Gh[1] * e1 - gm);
-    const T feq = W * a.rho0 + geq(a, k, dr, m);
+    const T s = T(3) * (Gh[0] * l.e[0] + Gh[1] * l.e[1] - gm);
+    const T feq = l.W * a.rho0 + geq_lane(l, a.inv_rho0, dr, m);
     T dg[2];
-    geq_dm(a, k, m, dg);
-    const T coef = b + c * s;  // dP/dgeq
-    bdr = w * coef * W;
-    bm[0] = w * (coef * dg[0] - c * T(3) * Gh[0] * a.inv_rho0 * feq);
-    bm[1] = w * (coef * dg[1] - c * T(3) * Gh[1] * a.inv_rho0 * feq);
-    bG[0] = w * c * T(3) * (e0 - m[0] * a.inv_rho0) * feq;
-    bG[1] = w * c * T(3) * (e1 - m[1] * a.inv_rho0) * feq;
+    geq_dm_lane(l, a.inv_rho0, m, dg);
+    const T cw = w * (b + c * s), fq = w * c * T(3) * feq;  // w dP/dgeq
+    bdr = wsum(cw * l.W);
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+        bm[i] = wsum(cw * dg[i] - fq * (Gh[i] * a.inv_rho0));
+        bG[i] = wsum(fq * (l.e[i] - m[i] * a.inv_rho0));
+    }
 }
 
 // ---- acceleration at cells and interfaces (reading R2) ----
@@ -254,162 +201,6 @@ template <class T>
 __device__ __forceinline__ void cell_Gh(const AdjParams<T> &a, int x, int y, T Gh[2]) {
     for (int c = 0; c < 2; c++) Gh[c] = (a.g[c] + field_at(a, c, x, y)) * a.ctc;
 }
-// Cells whose field the interface at position pos along d averages: wrapped on a periodic
-// axis, clamped at a wall (the one boundary cell).
-template <class T>
-__device__ __forceinline__ void face_cells(const AdjParams<T> &a, int d, int pos, int &lo, int &hi) {
-    const int nd = a.n[d];
-    lo = pos - 1;
-    hi = pos;
-    if (a.per[d]) {
-        if (lo < 0) lo += nd;
-        if (hi >= nd) hi -= nd;
-    } else {
-        if (lo < 0) lo = 0;
-        if (hi >= nd) hi = nd - 1;
-    }
-}
-template <class T>
-__device__ __forceinline__ void face_Gh(const AdjParams<T> &a, int d, int i, int j, T Gh[2]) {
-    int lo, hi;
-    face_cells(a, d, d == 0 ? i : j, lo, hi);
-    const int lx = d == 0 ? lo : i, ly = d == 1 ? lo : j, hx = d == 0 ? hi : i, hy = d == 1 ? hi : j;
-    for (int c = 0; c < 2; c++)
-        Gh[c] = (a.g[c] + T(0.5) * (field_at(a, c, lx, ly) + field_at(a, c, hx, hy))) * a.cthc;
-}
-
-// ---- forward state of one interface (steps 3-6), one velocity per lane ----
-template <class T>
-struct FaceLane {
-    T F, Fc;               // step-4 value of the lane's velocity (incoming ones replaced at a
-                           // wall, step 5) and its value at x_c (wall only)
-    T dr, m[2], Gh[2];     // step-6 moments and the interface acceleration
-    int wall, side, bb;    // bb: bounce-back wall (eq. (31))
-    T drc, mc[2];          // moments at x_c (wall only)
-    T ma[2];               // m_a of step 5 (wall only)
-};
-
-template <class T>
-__device__ __forceinline__ void face_forward_lane(const AdjParams<T> &a, int d, int i, int j, int k, bool act,
-                                                  FaceLane<T> &s) {
-    const T e0 = (T)L9::e(k, 0), e1 = (T)L9::e(k, 1);
-    s.F = act ? recon(a, d, i, j, k) : T(0);
-    const int pos = d == 0 ? i : j;
-    s.wall = !a.per[d] && (pos == 0 || pos == a.n[d]);
-    s.side = pos == 0 ? 0 : 1;
-    face_Gh(a, d, i, j, s.Gh);
-    s.Fc = T(0);
-    s.bb = s.wall && a.bc[2 * d + s.side] == DUGKS_BC_BOUNCE_BACK;
-    if (s.bb) {
-        // step 5, eq. (31): the incoming velocity takes its opposite's value (lane 8 - k of the
-        // half) plus 6 W_k e_k.m_w
-        const T Fo = __shfl_sync(0xffffu << (threadIdx.x & 16), s.F, Q - 1 - k, 16);
-        const int sgn = s.side == 0 ? -1 : 1;
-        const T *mw = a.mw[2 * d + s.side];
-        if (act && sgn * L9::e(k, d) < 0) s.F = Fo + T(6) * L9::wt<T>(k) * (e0 * mw[0] + e1 * mw[1]);
-    } else if (s.wall) {
-        // x_c: the boundary cell's opposite interface (reading R4)
-        const int sh = s.side == 0 ? 1 : -1;
-        const int ci = d == 0 ? i + sh : i, cj = d == 1 ? j + sh : j;
-        s.Fc = act ? recon(a, d, ci, cj, k) : T(0);
-        T Ghc[2];
-        face_Gh(a, d, ci, cj, Ghc);
-        s.drc = wsum(s.Fc);
-        s.mc[0] = wsum(e0 * s.Fc) + a.rho0 * Ghc[0] * a.wface;
-        s.mc[1] = wsum(e1 * s.Fc) + a.rho0 * Ghc[1] * a.wface;
-        const int wid = 2 * d + s.side;
-        const bool vel = a.bc[wid] == DUGKS_BC_NEQ_VELOCITY;
-        const T dra = vel ? s.drc : a.drw[wid] + a.drw1[wid] * a.cwh;
-        s.ma[0] = vel ? a.mw[wid][0] : s.mc[0];
-        s.ma[1] = vel ? a.mw[wid][1] : s.mc[1];
-        const int sgn = s.side == 0 ? -1 : 1;
-        if (act && sgn * L9::e(k, d) < 0) s.F = geq(a, k, dra, s.ma) + s.Fc - geq(a, k, s.drc, s.mc);
-    }
-    s.dr = wsum(s.F);
-    s.m[0] = wsum(e0 * s.F) + a.rho0 * s.Gh[0] * a.wface;
-    s.m[1] = wsum(e1 * s.F) + a.rho0 * s.Gh[1] * a.wface;
-}
-
-// Adjoint of steps 5-9 at interface (d, i, j) for lambda', velocity k of this lane. Fb:
-// dL/d(step-4 value), zero for a velocity the wall replaces; Gb: dL/dGh of the interface
-// (the same in every lane). At a wall also what flows to the step-4 value and Gh of x_c
-// (Fcb, Gcb) and to the wall velocity (Wb).
-template <class T>
-__device__ __forceinline__ void face_adjoint_lane(const AdjParams<T> &a, int d, int i, int j, int k, bool act,
-                                                  T &Fb, T Gb[2], T &Fcb, T Gcb[2], T Wb[2], int &wall) {
-    FaceLane<T> s;
-    face_forward_lane(a, d, i, j, k, act, s);
-    wall = s.wall;
-    const int64_t nc = ncell(a);
-    const int pos = d == 0 ? i : j, nd = a.n[d];
-    const T e0 = (T)L9::e(k, 0), e1 = (T)L9::e(k, 1);
-    // steps 8-9: velocity k of this interface enters the update of its low cell with
-    // -2 kappa e_d and of its high cell with +2 kappa e_d
-    const bool haslo = pos > 0, hashi = pos < nd;
-    const int plo = pos > 0 ? pos - 1 : nd - 1, phi_c = pos < nd ? pos : 0;
-    const int64_t clo = d == 0 ? plo + (int64_t)a.n[0] * j : i + (int64_t)a.n[0] * plo;
-    const int64_t chi = d == 0 ? phi_c + (int64_t)a.n[0] * j : i + (int64_t)a.n[0] * phi_c;
-    const int ed = L9::e(k, d);
-    T v = T(0);
-    if (act && ed) {
-        if (haslo) v -= a.lam1[k * nc + clo];
-        if (hashi) v += a.lam1[k * nc + chi];
-    }
-    const T fbar = a.two_kappa * (T)ed * v;
-    // step 7 (eq. (20)) at the step-6 moments, then step 6
-    T bdr, bm[2], bG[2];
-    relax_T_one(a, k, fbar, s.dr, s.m, s.Gh, a.b7, a.c7, bdr, bm, bG);
-    bdr = wsum(bdr);
-    bm[0] = wsum(bm[0]);
-    bm[1] = wsum(bm[1]);
-    Gb[0] = wsum(bG[0]) + a.rho0 * a.wface * bm[0];
-    Gb[1] = wsum(bG[1]) + a.rho0 * a.wface * bm[1];
-    Fb = act ? (T(1) - a.b7) * fbar + bdr + e0 * bm[0] + e1 * bm[1] : T(0);
-    Fcb = T(0);
-    Gcb[0] = Gcb[1] = T(0);
-    Wb[0] = Wb[1] = T(0);
-    if (!wall) return;
-    if (s.bb) {
-        // step 5, eq. (31): F_k = F_-k + 6 W_k e_k.m_w for incoming k: the weight of an
-        // incoming velocity passes to its opposite (lane 8 - k) and to u_w
-        const int sgn = s.side == 0 ? -1 : 1;
-        const bool incoming = act && sgn * ed < 0;
-        const T w = incoming ? Fb : T(0);
-        const T back = __shfl_sync(0xffffu << (threadIdx.x & 16), w, Q - 1 - k, 16);
-        Fb = (incoming ? T(0) : Fb) + back;
-        const T c6 = T(6) * L9::wt<T>(k) * w * a.dmw;
-        Wb[0] = wsum(c6 * e0);
-        Wb[1] = wsum(c6 * e1);
-        return;
-    }
-    // step 5 (eq. (32)): F_k = geq_k(drho_a, m_a) + Fc_k - geq_k(drho_c, m_c), incoming k.
-    // Velocity condition: drho_a = drho_c (the W_k terms cancel), m_a from u_w.
-    // Pressure condition: m_a = m_c (the m terms cancel), drho_a fixed.
-    const int wid = 2 * d + s.side;
-    const bool vel = a.bc[wid] == DUGKS_BC_NEQ_VELOCITY;
-    const int sgn = s.side == 0 ? -1 : 1;
-    const bool incoming = act && sgn * ed < 0;
-    const T w = incoming ? Fb : T(0);
-    if (incoming) Fb = T(0);
-    Fcb = w;
-    T bdrc = T(0), bmc[2] = {T(0), T(0)};
-    if (vel) {
-        T da[2], dc[2];
-        geq_dm(a, k, s.ma, da);
-        geq_dm(a, k, s.mc, dc);
-        Wb[0] = wsum(w * da[0] * a.dmw);
-        Wb[1] = wsum(w * da[1] * a.dmw);
-        bmc[0] = -wsum(w * dc[0]);
-        bmc[1] = -wsum(w * dc[1]);
-    } else {
-        bdrc = -wsum(w * L9::wt<T>(k));
-    }
-    // step 6 at x_c
-    if (act) Fcb += bdrc + e0 * bmc[0] + e1 * bmc[1];
-    Gcb[0] = a.rho0 * a.wface * bmc[0];
-    Gcb[1] = a.rho0 * a.wface * bmc[1];
-}
-
 // ---- fast paths: interfaces and cells whose stencils lie inside the domain, away from
 // walls and periodic seams (no ghosts, images, NEQ or x_c coupling). Same arithmetic as the
 // general path, with compile-time velocities and direct neighbour reads. ----
@@ -467,26 +258,22 @@ __host__ __device__ inline int64_t rect_count(const Rect &r) {
     return rect_empty(r) ? 0 : (int64_t)(r.x1 - r.x0 + 1) * (r.y1 - r.y0 + 1);
 }
 __host__ __device__ inline int64_t frame_count(const Rect &r) { return (int64_t)r.W * r.H - rect_count(r); }
-// The t-th element (row-major) of the index space outside the fast rectangle.
-__device__ inline void frame_at(const Rect &r, int64_t t, int &x, int &y) {
-    if (rect_empty(r)) {
-        x = (int)(t % r.W);
-        y = (int)(t / r.W);
-        return;
-    }
-    const int64_t below = (int64_t)r.y0 * r.W, above = (int64_t)(r.H - 1 - r.y1) * r.W;
-    if (t < below) {
-        x = (int)(t % r.W);
-        y = (int)(t / r.W);
-    } else if (t < below + above) {
-        t -= below;
-        x = (int)(t % r.W);
-        y = r.y1 + 1 + (int)(t / r.W);
+// The t-th element (row-major) of the index space outside the fast rectangle. 32-bit counts: the
+// sweep's some 45 values per cell leave room for fewer than 2^31 cells.
+__device__ inline void frame_at(const Rect &r, unsigned t, int &x, int &y) {
+    const unsigned W = (unsigned)r.W;
+    const bool none = rect_empty(r);
+    const unsigned below = none ? ~0u : (unsigned)r.y0 * W, above = none ? 0u : (unsigned)(r.H - 1 - r.y1) * W;
+    if (t < below || t - below < above) {
+        y = (int)(t / W);
+        x = (int)(t - (unsigned)y * W);
+        if (t >= below) y += r.y1 + 1 - r.y0;
     } else {
         t -= below + above;
-        const int side = r.x0 + (r.W - 1 - r.x1);  // frame columns of a middle row
-        y = r.y0 + (int)(t / side);
-        const int c = (int)(t % side);
+        const unsigned side = (unsigned)(r.x0 + (r.W - 1 - r.x1));  // frame columns of a middle row
+        const unsigned row = t / side;
+        const int c = (int)(t - row * side);
+        y = r.y0 + (int)row;
         x = c < r.x0 ? c : r.x1 + 1 + (c - r.x0);
     }
 }
@@ -584,7 +371,7 @@ __device__ __forceinline__ void cell_fast(const AdjParams<T> &a, int x, int y, i
 template <class T>
 __device__ __noinline__ void fwd_cell(const AdjParams<T> &a, const T *state, T ctc, T *mom, int64_t c) {
     const int64_t nc = ncell(a);
-    const int x = (int)(c % a.n[0]), y = (int)(c / a.n[0]);
+    const int y = (int)((unsigned)c / (unsigned)a.n[0]), x = (int)c - y * a.n[0];
     T g[Q], Gh[2], dr, m[2];
 #pragma unroll
     for (int k = 0; k < Q; k++) g[k] = state[k * a.dstride + (int64_t)y * a.px + x];
@@ -610,50 +397,146 @@ __global__ void __launch_bounds__(256) adj_cells_fwd(const AdjParams<T> a) {
         fwd_cell(a, a.state, a.ctc, a.mom, c);
 }
 
-// The t-th interface of the frame of both axes (walls: NEQ and dL/du_w; x_c interfaces;
-// periodic seams), one velocity per lane of the calling half-warp.
+// The t-th interface of the frame of both axes, one velocity per lane of the calling half-warp. The
+// interface next to a wall is x_c of the wall's (reading R4) and has the wall's item as well: both
+// take their step-4 values from the same two cells of each line, and what the wall passes to x_c
+// (step 5) stays in the lane. The time of this kernel and of the cells' is the latency of one frame item
+// wherever the interior is small (512 x 256 channel: 30.6 us per reverse step when a wall, an
+// x_c and a corner each formed their neighbours' values anew, 13 us of each kernel in the frame
+// alone; now 22).
 template <class T>
-__device__ __noinline__ void faces_frame_item(const AdjParams<T> &a, int64_t t) {
+__device__ __noinline__ void faces_frame_item(const AdjParams<T> &a, unsigned t) {
     const Rect r0 = face_rect(0, a.n[0], a.n[1], a.per[0], a.per[1]);
     const Rect r1 = face_rect(1, a.n[0], a.n[1], a.per[0], a.per[1]);
-    const int64_t c0 = frame_count(r0);
-    const int lane = half_lane();
-    const bool act = lane < Q;
-    const int k = act ? lane : 0;
+    const unsigned c0 = (unsigned)frame_count(r0);
     const int d = t < c0 ? 0 : 1;
     int i, j;
     frame_at(d == 0 ? r0 : r1, d == 0 ? t : t - c0, i, j);
-    const int64_t f = fidx(a, d, i, j);
-    const int pos = d == 0 ? i : j, nd = a.n[d];
-    T Fb, Gb[2], Fcb, Gcb[2], Wb[2];
-    int wall;
-    face_adjoint_lane(a, d, i, j, k, act, Fb, Gb, Fcb, Gcb, Wb, wall);
-    const int wbc = a.bc[2 * d + (pos == 0 ? 0 : 1)];
-    if (wall && a.dW && lane == 0 && (wbc == DUGKS_BC_NEQ_VELOCITY || wbc == DUGKS_BC_BOUNCE_BACK)) {
-        const int64_t slot = d == 0 ? (pos == 0 ? 0 : a.n[1]) + j : 2 * (int64_t)a.n[1] + (pos == 0 ? 0 : a.n[0]) + i;
-        a.dW[2 * slot] += (double)Wb[0];
-        a.dW[2 * slot + 1] += (double)Wb[1];
-    }
-    // this interface is x_c of the wall interface at 0 (pos == 1) and/or at nd (pos == nd - 1)
-    if (!a.per[d]) {
-        for (int sd = 0; sd < 2; sd++) {
-            if (pos != (sd == 0 ? 1 : nd - 1)) continue;
-            const int wp = sd == 0 ? 0 : nd;
-            T wFb, wGb[2], wFcb, wGcb[2], wWb[2];
-            int ww;
-            face_adjoint_lane(a, d, d == 0 ? wp : i, d == 1 ? wp : j, k, act, wFb, wGb, wFcb, wGcb, wWb, ww);
-            Fb += wFcb;
-            Gb[0] += wGcb[0];
-            Gb[1] += wGcb[1];
+    const int n = d == 0 ? a.n[0] : a.n[1], nt = d == 0 ? a.n[1] : a.n[0];
+    const int per = d == 0 ? a.per[0] : a.per[1], pert = d == 0 ? a.per[1] : a.per[0];
+    const int pos = d == 0 ? i : j, tp = d == 0 ? j : i;
+    if (!per && (pos == 0 || pos == n)) return;  // a wall: its x_c's item makes it
+    const LaneVel<T> l;
+    const int lane = half_lane(), ien = d == 0 ? l.ie[0] : l.ie[1];
+    const T en = d == 0 ? l.e[0] : l.e[1], et = d == 0 ? l.e[1] : l.e[0];
+    const int64_t nc = ncell(a);
+    const unsigned nx = (unsigned)a.n[0], sn = d == 0 ? 1u : nx, st = d == 0 ? nx : 1u;
+    // the two cells, and their tangential neighbours
+    const unsigned lo = sn * (unsigned)(pos > 0 ? pos - 1 : n - 1), hi = sn * (unsigned)(pos < n ? pos : 0);
+    const unsigned own = st * (unsigned)tp;
+    int cp[2], cm[2];
+    T wp[2], wm[2];
+    ext2<T>(tp + 1, nt, pert, cp, wp);
+    ext2<T>(tp - 1, nt, pert, cm, wm);
+    const T *ph = a.phi + l.k * nc, *lam = a.lam1 + l.k * nc;
+    auto line = [&](unsigned c, T &v, T &dv) __attribute__((always_inline)) {
+        v = ph[c + own];
+        dv = (wp[0] * ph[c + st * (unsigned)cp[0]] + wp[1] * ph[c + st * (unsigned)cp[1]]) -
+             (wm[0] * ph[c + st * (unsigned)cm[0]] + wm[1] * ph[c + st * (unsigned)cm[1]]);
+        if (!l.act) v = dv = T(0);
+    };
+    T A, dA, B, dB;
+    line(lo, A, dA);
+    line(hi, B, dB);
+    const T lamA = l.act ? lam[lo + own] : T(0), lamB = l.act ? lam[hi + own] : T(0);
+    T fA[2] = {T(0), T(0)}, fB[2] = {T(0), T(0)};
+    if (a.field) {
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            fA[c] = (T)a.field[c * nc + lo + own];
+            fB[c] = (T)a.field[c * nc + hi + own];
         }
     }
-    T *fb = a.fb[d], *gb = a.gb[d];
+    const T k4 = T(0.25) * a.kappa * et, kn = a.kappa * en, rw = a.rho0 * a.wface;
     const int64_t nf = nface(a, d);
-    if (act) fb[k * nf + f] = Fb;
-    if (lane == 0) {
-        gb[f] = Gb[0];
-        gb[nf + f] = Gb[1];
+    T *fb = a.fb[d] + l.k * nf, *gb = a.gb[d];
+    auto face_at = [&](int p) __attribute__((always_inline)) { return d == 0 ? fidx(a, 0, p, tp) : fidx(a, 1, tp, p); };
+    auto store = [&](int64_t f, T Fb, T G0, T G1) __attribute__((always_inline)) {
+        if (l.act) fb[f] = Fb;
+        if (lane < 2) gb[lane * nf + f] = lane ? G1 : G0;
+    };
+    // ---- the interface itself: steps 3-7 forward, then steps 9-6 backward. Steps 8-9: velocity k
+    // enters the update of the low cell with -2 kappa e_d and of the high cell with +2 kappa e_d ----
+    const T F = T(0.5) * (A + B) - kn * (B - A) - k4 * (dA + dB);
+    T Gh[2], m[2], Gb[2], bdr, bm[2];
+#pragma unroll
+    for (int c = 0; c < 2; c++) Gh[c] = (a.g[c] + T(0.5) * (fA[c] + fB[c])) * a.cthc;
+    const T dr = wsum(F);
+#pragma unroll
+    for (int c = 0; c < 2; c++) m[c] = wsum(l.e[c] * F) + rw * Gh[c];
+    const T fbar = a.two_kappa * en * ((pos < n ? lamB : T(0)) - (pos > 0 ? lamA : T(0)));
+    relax_T_lane(a, l, fbar, dr, m, Gh, a.b7, a.c7, bdr, bm, Gb);
+    T Fb = (T(1) - a.b7) * fbar + bdr + l.e[0] * bm[0] + l.e[1] * bm[1];
+#pragma unroll
+    for (int c = 0; c < 2; c++) Gb[c] += rw * bm[c];
+    // ---- the wall interfaces whose x_c it is ----
+#pragma unroll 1
+    for (int sd = 0; sd < 2; sd++) {
+        if (per || pos != (sd == 0 ? 1 : n - 1)) continue;
+        const int wid = 2 * d + sd, type = a.bc[wid];
+        const T sg = sd == 0 ? T(1) : T(-1);  // the incoming velocities' e_d
+        const T C = sd == 0 ? A : B, dC = sd == 0 ? dA : dB;  // the wall's cell; its ghost (step 2) is 2 C - other
+        const T G = T(2) * C - (sd == 0 ? B : A), dG = T(2) * dC - (sd == 0 ? dB : dA);
+        const bool incoming = l.act && (sd == 0 ? ien > 0 : ien < 0), bb = type == DUGKS_BC_BOUNCE_BACK;
+        const bool vel = type == DUGKS_BC_NEQ_VELOCITY;
+        T Fw = T(0.5) * (G + C) - kn * sg * (C - G) - k4 * (dG + dC);
+        const unsigned mask = 0xffffu << (threadIdx.x & 16);
+        const int64_t slot = d == 0 ? (sd == 0 ? 0 : a.n[1]) + j : 2 * (int64_t)a.n[1] + (sd == 0 ? 0 : a.n[0]) + i;
+        const bool wantW = a.dW && (bb || vel) && lane < 2;
+        const double dW0 = wantW ? a.dW[2 * slot + lane] : 0.0;
+        const T mw[2] = {a.mw[wid][0], a.mw[wid][1]};
+        T Gw[2], mwf[2], Gwb[2], Wb[2], ma[2];
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            Gw[c] = (a.g[c] + (sd == 0 ? fA[c] : fB[c])) * a.cthc;
+            ma[c] = vel ? mw[c] : m[c];
+        }
+        // step 5: eq. (31), or eq. (32) with drho_a, m_a of a velocity or a pressure condition
+        const T Fo = __shfl_sync(mask, Fw, Q - 1 - l.k, 16);
+        const T dra = vel ? dr : a.drw[wid] + a.drw1[wid] * a.cwh;
+        const T Fin = bb ? Fo + T(6) * l.W * (l.e[0] * mw[0] + l.e[1] * mw[1])
+                         : geq_lane(l, a.inv_rho0, dra, ma) + F - geq_lane(l, a.inv_rho0, dr, m);
+        if (incoming) Fw = Fin;
+        const T drw = wsum(Fw);
+#pragma unroll
+        for (int c = 0; c < 2; c++) mwf[c] = wsum(l.e[c] * Fw) + rw * Gw[c];
+        const T fw = a.two_kappa * en * (sd == 0 ? lamA : -lamB);
+        T bd, b[2];
+        relax_T_lane(a, l, fw, drw, mwf, Gw, a.b7, a.c7, bd, b, Gwb);
+        T Fwb = (T(1) - a.b7) * fw + bd + l.e[0] * b[0] + l.e[1] * b[1];
+        // step 5 backward: the weight of an incoming velocity passes to its opposite and u_w (eq. (31)),
+        // or to x_c's value and moments and to u_w (the W_k terms of a velocity condition and the m terms of a
+        // pressure condition cancel)
+        const T w = incoming ? Fwb : T(0);
+        if (incoming) Fwb = T(0);
+        T dw[2];
+        if (bb) {
+            Fwb += __shfl_sync(mask, w, Q - 1 - l.k, 16);
+#pragma unroll
+            for (int c = 0; c < 2; c++) dw[c] = T(6) * l.W * l.e[c];
+        } else {
+            T xd = T(0), xm[2] = {T(0), T(0)};
+            geq_dm_lane(l, a.inv_rho0, mw, dw);
+            if (vel) {
+                T dc[2];
+                geq_dm_lane(l, a.inv_rho0, m, dc);
+#pragma unroll
+                for (int c = 0; c < 2; c++) xm[c] = -wsum(w * dc[c]);
+            } else {
+                xd = -wsum(w * l.W);
+            }
+            Fb += w + xd + l.e[0] * xm[0] + l.e[1] * xm[1];
+#pragma unroll
+            for (int c = 0; c < 2; c++) Gb[c] += rw * xm[c];
+        }
+        if (a.dW && (bb || vel)) {
+#pragma unroll
+            for (int c = 0; c < 2; c++) Wb[c] = wsum(w * dw[c] * a.dmw);
+            if (wantW) a.dW[2 * slot + lane] = dW0 + (double)(lane ? Wb[1] : Wb[0]);
+        }
+        store(face_at(sd == 0 ? 0 : n), Fwb, Gwb[0] + rw * b[0], Gwb[1] + rw * b[1]);
     }
+    store(face_at(pos), Fb, Gb[0], Gb[1]);
 }
 
 // Every interface of both axes in one launch of 128-thread blocks: the frame blocks first
@@ -663,7 +546,7 @@ template <class T>
 __global__ void __launch_bounds__(128, 6) adj_faces_all(const AdjParams<T> a, int64_t nframe, int nfb, int nt0,
                                                          int tx0, int tx1) {
     if ((int)blockIdx.x < nfb) {
-        const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+        const unsigned t = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
         if (t < nframe) faces_frame_item(a, t);
         return;
     }
@@ -679,92 +562,109 @@ __global__ void __launch_bounds__(128, 6) adj_faces_all(const AdjParams<T> a, in
     else face_fast<T, 1>(a, i, j, f, nface(a, 1));
 }
 
-// dL/dGh summed over the interfaces whose acceleration averages cell (x, y), with the
-// averaging weights (1/2 per side; the clamped wall interface takes the cell twice).
+// Transposes of the reconstruction and of step 2 along one axis, for the cell at x of n: the (at most
+// four) interfaces across the axis whose step-4 values it enters as one of the two cells, directly or
+// through a ghost or an image, as weights of the normal part (h -+ kappa e: w1), of the
+// tangential part (w2) and of the interface acceleration (wg; reading R2); and its rows as a
+// tangential neighbour, above, own (through a ghost) and below, with weights t.
 template <class T>
-__device__ __forceinline__ T face_G_T(const AdjParams<T> &a, int comp, int x, int y) {
-    T s = T(0);
-    for (int d = 0; d < 2; d++) {
-        const int pc = d == 0 ? x : y, nd = a.n[d];
-        int cand[4], nc = 0;
-        cand[nc++] = pc;
-        cand[nc++] = pc + 1;
-        if (a.per[d] && nd > 1) {  // the interfaces across the periodic seam
-            if (pc == nd - 1) cand[nc++] = 0;
-            if (pc == 0) cand[nc++] = nd;
-        }
-        const int64_t nf = nface(a, d);
-        for (int u = 0; u < nc; u++) {
-            int lo, hi;
-            face_cells(a, d, cand[u], lo, hi);
-            const T w = (lo == pc ? T(0.5) : T(0)) + (hi == pc ? T(0.5) : T(0));
-            if (w != T(0)) {
-                const int i = d == 0 ? cand[u] : x, j = d == 1 ? cand[u] : y;
-                s += w * a.gb[d][comp * nf + fidx(a, d, i, j)];
-            }
-        }
+struct AxisT {
+    int f[4], row[3];  // f < 0: absent
+    T w1[4], w2[4], wg[4], t[3];
+    __device__ __forceinline__ AxisT(int x, int n, int per, T ke) {
+        const T hp = T(0.5) + ke, hm = T(0.5) - ke;
+        const bool lo = !per && x == 0, hi = !per && x == n - 1, lo1 = !per && x == 1, hi1 = !per && x == n - 2;
+        const bool pl = per && x == 0, ph = per && x == n - 1;
+        f[0] = x;
+        w1[0] = hm + (lo ? T(2) * hp : T(0));
+        w2[0] = lo ? T(3) : T(1);
+        wg[0] = lo ? T(1) : T(0.5);
+        f[1] = x + 1;
+        w1[1] = hp + (hi ? T(2) * hm : T(0));
+        w2[1] = hi ? T(3) : T(1);
+        wg[1] = hi ? T(1) : T(0.5);
+        f[2] = lo1 || ph ? 0 : -1;
+        w1[2] = ph ? hp : -hp;
+        w2[2] = ph ? T(1) : T(-1);
+        wg[2] = ph ? T(0.5) : T(0);
+        f[3] = hi1 || pl ? n : -1;
+        w1[3] = pl ? hm : -hm;
+        w2[3] = pl ? T(1) : T(-1);
+        wg[3] = pl ? T(0.5) : T(0);
+        row[0] = x + 1 < n ? x + 1 : (per ? 0 : x);
+        row[1] = x;
+        row[2] = x > 0 ? x - 1 : (per ? n - 1 : x);
+        t[0] = hi ? T(0) : (hi1 ? T(2) : T(1));
+        t[1] = (lo ? T(2) : T(0)) - (hi ? T(2) : T(0));
+        t[2] = lo ? T(0) : (lo1 ? T(-2) : T(-1));
     }
-    return s;
-}
+};
 
 // The t-th frame cell (cells whose stencil meets a wall ghost, a periodic image or a
-// wall-clamped interface acceleration), one velocity per lane of the calling half-warp.
+// wall-clamped interface acceleration), one velocity per lane of the calling half-warp. Every
+// load's address is known at the start.
 template <class T>
-__device__ __noinline__ void cells_frame_item(const AdjParams<T> &a, int64_t t) {
-    const int64_t nc = ncell(a);
+__device__ __noinline__ void cells_frame_item(const AdjParams<T> &a, unsigned t) {
+    const int64_t nc = ncell(a), n0 = nface(a, 0), n1 = nface(a, 1);
     const Rect r = cell_rect(a.n[0], a.n[1], a.per[0], a.per[1]);
-    const int lane = half_lane();
-    const bool act = lane < Q;
-    const int k = act ? lane : 0;
     int x, y;
     frame_at(r, t, x, y);
-    const int64_t c = x + (int64_t)a.n[0] * y;
-    int ux[3], uy[3];
-    T wx[3], wy[3];
-    const int nux = ext_users<T>(x, a.n[0], a.per[0], ux, wx);
-    const int nuy = ext_users<T>(y, a.n[1], a.per[1], uy, wy);
-    // adjoint of fbar+ of this cell: eq. (25) (4/3 fbar+) and every interface value
-    // reconstructed from it, directly or through a ghost / periodic image
-    const T l1 = act ? a.lam1[k * nc + c] : T(0);
-    T pb = T(0);
-    if (act) {
-        T v = T(4) / T(3) * l1;
-        for (int p = 0; p < nux; p++)
-            for (int q = 0; q < nuy; q++) v += wx[p] * wy[q] * recon_T(a, k, ux[p], uy[q]);
-        pb = v;
-    }
-    // step 1 (eq. (24)) and the cell moments (eq. (27))
+    const LaneVel<T> l;
+    const int lane = half_lane();
+    const unsigned nx = (unsigned)a.n[0], c = (unsigned)x + nx * (unsigned)y;
+    const AxisT<T> ax(x, a.n[0], a.per[0], a.kappa * l.e[0]), ay(y, a.n[1], a.per[1], a.kappa * l.e[1]);
     const T dr = a.mom[c];
     const T m[2] = {a.mom[nc + c], a.mom[2 * nc + c]};
     T Gh[2];
     cell_Gh(a, x, y, Gh);
-    T bdr, bm[2], bG[2];
-    relax_T_one(a, k, pb, dr, m, Gh, a.b1, a.c1, bdr, bm, bG);
-    bdr = wsum(bdr);
-    bm[0] = wsum(bm[0]);
-    bm[1] = wsum(bm[1]);
-    bG[0] = wsum(bG[0]);
-    bG[1] = wsum(bG[1]);
-    if (act)
-        a.lam0[k * nc + c] = -l1 / T(3) + (T(1) - a.b1) * pb + bdr + (T)L9::e(k, 0) * bm[0] + (T)L9::e(k, 1) * bm[1];
-    if (a.dG && lane < 2) {
-        const int comp = lane;
-        const T sv = (bG[comp] + a.rho0 * a.wcell * bm[comp]) * a.ctc + face_G_T(a, comp, x, y) * a.cthc;
-        a.dG[comp * nc + c] += (double)sv;
+    const T l1 = a.lam1[l.k * nc + c];
+    const int comp = lane & 1;
+    const bool wantG = a.dG && lane < 2;
+    const double g0 = wantG ? a.dG[comp * nc + c] : 0.0;
+    // adjoint of fbar+ of this cell: eq. (25) (4/3 fbar+) and the interface values it enters
+    const T *f0 = a.fb[0] + l.k * n0, *f1 = a.fb[1] + l.k * n1;
+    const T *g0x = a.gb[0] + comp * n0, *g1y = a.gb[1] + comp * n1;
+    const T q = T(0.25) * a.kappa;
+    T pb = T(4) / T(3) * l1, gs = T(0);
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+        if (s >= 2 && ax.f[s] < 0) continue;
+        const T *p = f0 + ax.f[s];
+        const unsigned sr = nx + 1, o = sr * (unsigned)y;
+        const T v = p[o], u = ay.t[0] * p[sr * (unsigned)ay.row[0]] + ay.t[1] * v + ay.t[2] * p[sr * (unsigned)ay.row[2]];
+        pb += ax.w1[s] * v + q * l.e[1] * ax.w2[s] * u;
+        if (wantG) gs += ax.wg[s] * g0x[ax.f[s] + o];
     }
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+        if (s >= 2 && ay.f[s] < 0) continue;
+        const T *p = f1 + (int64_t)nx * ay.f[s];
+        const T v = p[x], u = ax.t[0] * p[ax.row[0]] + ax.t[1] * v + ax.t[2] * p[ax.row[2]];
+        pb += ay.w1[s] * v + q * l.e[0] * ay.w2[s] * u;
+        if (wantG) gs += ay.wg[s] * g1y[(int64_t)nx * ay.f[s] + x];
+    }
+    if (!l.act) pb = T(0);
+    // step 1 (eq. (24)) and the cell moments (eq. (27))
+    T bdr, bm[2], bG[2];
+    relax_T_lane(a, l, pb, dr, m, Gh, a.b1, a.c1, bdr, bm, bG);
+    if (l.act) a.lam0[l.k * nc + c] = -l1 / T(3) + (T(1) - a.b1) * pb + bdr + l.e[0] * bm[0] + l.e[1] * bm[1];
+    if (wantG)
+        a.dG[comp * nc + c] = g0 + (double)(((comp ? bG[1] : bG[0]) + a.rho0 * a.wcell * (comp ? bm[1] : bm[0])) * a.ctc +
+                                            gs * a.cthc);
 }
 
 // All cells in one launch of 128-thread blocks: frame blocks first (a half-warp per frame cell),
 // then 32 x 4 tiles of the fast rectangle (tx x ty blocks).
 // With a.nstate set, the blocks then recompute the next reverse step's fbar+ and moments,
-// one cell per thread, the interior tiles first (the frame blocks are the longest): this
+// one cell per thread in the blocks' order, so that the blocks of a last, partial wave have none
+// (512 x 256: 3% of a reverse step against giving them to the interior tiles first): this
 // step's interfaces no longer read a.phi, and each cell's moments go to the other buffer, so
 // no block reads what another overwrites.
 template <class T>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 7 : 5) adj_cells_all(const AdjParams<T> a, int nfb, int tx, int ty) {
     const Rect r = cell_rect(a.n[0], a.n[1], a.per[0], a.per[1]);
     if ((int)blockIdx.x < nfb) {  // eight frame cells per block, one per half-warp
-        const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 4);
+        const unsigned t = blockIdx.x * 8 + (threadIdx.x >> 4);
         if (t < frame_count(r)) cells_frame_item(a, t);
     } else {
         const int b = blockIdx.x - nfb;
@@ -773,9 +673,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 7 : 5) adj_cells_all(con
     }
     if (a.nstate) {
         const int64_t nc = ncell(a);
-        const int nb = (int)gridDim.x, bi = (int)blockIdx.x;
-        const int rb = bi >= nfb ? bi - nfb : bi + (nb - nfb);  // tiles take blocks 0 .. nb - nfb - 1
-        for (int64_t c = rb * (int64_t)blockDim.x + threadIdx.x; c < nc; c += (int64_t)nb * blockDim.x)
+        for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x)
             fwd_cell(a, a.nstate, a.nctc, a.nmom, c);
     }
 }
