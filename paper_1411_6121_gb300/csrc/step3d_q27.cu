@@ -1,5 +1,5 @@
 // step3d_q27.cu -- the 3D throughput kernels instantiated for D3Q27 (the paper's 3D velocity set,
-// Sec. 2.3), F32/BF16/F16 storage: the warp-specialised one (dugks_step3d_ws.cuh, the default) and
+// Sec. 2.3), F32/BF16/F16 storage: the warp-specialised one (dugks_step3d_ws27.cuh, the default) and
 // the non-specialised one (dugks_step3d.cuh, 32 x 8 columns per CTA; at 27 velocities its TMA
 // stages do not fit beside the ring, so every plane is loaded directly and the tensor map is
 // unused).
@@ -7,7 +7,7 @@
 
 #include "dugks_internal.h"
 #include "dugks_step3d.cuh"
-#include "dugks_step3d_ws.cuh"
+#include "dugks_step3d_ws27.cuh"
 
 namespace dugks {
 
