@@ -34,7 +34,7 @@ cudaError_t launch_step_q9(const StepParams &p, int store, int tx, int ty, cudaS
 cudaError_t launch_step_q19(const StepParams &p, int store, int tx, int ty, cudaStream_t stream);
 cudaError_t launch_step_q27(const StepParams &p, int store, int tx, int ty, cudaStream_t stream);
 // Throughput kernels for D3Q19 and D3Q27 with F32/BF16/F16 storage: ry 0 the warp-specialised one
-// (dugks_step3d_ws.cuh), else the non-specialised one (dugks_step3d.cuh) with ry CTA rows (D3Q27: 8).
+// (dugks_step3d_ws.cuh, dugks_step3d_ws27.cuh), else the non-specialised one (dugks_step3d.cuh) with ry CTA rows (D3Q27: 8).
 cudaError_t launch_step3d_q19(const StepParams &p, int store, int ry, cudaStream_t stream);
 cudaError_t launch_step3d_q27(const StepParams &p, int store, int ry, cudaStream_t stream);
 // Throughput kernel for D2Q9 with F32/BF16/F16 storage (dugks_step2d.cuh; BF16:
