@@ -132,11 +132,14 @@ __device__ __forceinline__ V unpack2(uint32_t w) {  // two F16 values
     return mul(__half22float2(*reinterpret_cast<const __half2 *>(&w)), bc(F16_UNSCALE));
 }
 
-// The two values as stored, rounded stochastically (store_state_pair): r[15:0] rounds the first,
-// which goes to the low half.
-__device__ __forceinline__ uint32_t f16_pair(V v, uint32_t r) {
+// The two values as stored, each rounded as store_state rounds it (the low 13 bits of its random bits
+// r added below the kept significand, then truncated), the first in the low half.
+__device__ __forceinline__ uint32_t f16_pair(V v, uint32_t r0, uint32_t r1) {
+    const V t = mul(v, bc(F16_SCALE));
     uint32_t d;
-    asm("cvt.rs.satfinite.f16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.y * F16_SCALE), "f"(v.x * F16_SCALE), "r"(r));
+    asm("cvt.rz.f16x2.f32 %0, %1, %2;"
+        : "=r"(d)
+        : "f"(__uint_as_float(__float_as_uint(t.y) + (r1 & 0x1fffu))), "f"(__uint_as_float(__float_as_uint(t.x) + (r0 & 0x1fffu))));
     return d;
 }
 
@@ -770,12 +773,12 @@ __device__ __forceinline__ void tile(const StepParams &p, V *sm, int x0, int y0)
             for (int k = 0; k < 9; k++) o[k * p.dstride] = u0[k].x;
         }
     } else {
-        // F16: one conversion rounds the lane's two cells stochastically, fed by one random word (some
-        // 150 instructions less than rounding each in software)
-        const CellRandom rnd(seed, off);
+        // F16: each value takes the random bits that it has in every kernel (CellRandom), so the noise of a
+        // run does not depend on the kernel; one conversion truncates the lane's two cells
+        const CellRandom rnd0(seed, off), rnd1(seed, off + 1);
         sfor<9>([&](auto kc) {
             constexpr int k = kc;
-            const uint32_t w = f16_pair(u0[k], rnd.template word<k>());
+            const uint32_t w = f16_pair(u0[k], rnd0.template bits<k>(), rnd1.template bits<k>());
             if (upd1) *reinterpret_cast<uint32_t *>(o + k * p.dstride) = w;
             else if (upd0) o[k * p.dstride] = __ushort_as_half((unsigned short)(w & 0xffffu));
         });

@@ -1111,8 +1111,9 @@ __global__ void __launch_bounds__(512, 1)
                 }
                 // eq. (16): f~(t+dt) = f~+ - dt/|V| flux
                 const float2 v = __fadd2_rn(u, __ffma2_rn(f2(tk * w, tk * w), n, __fmul2_rn(f2(lk, lk), l)));
-                store_state_pair<S>(dst + j * p.dstride + off, v.x, dst + (Q - 1 - j) * p.dstride + off, v.y,
-                                    sizeof(S) == 2 ? rnd.template word<j>() : 0u);
+                // the random bits that each value has in every kernel of the set
+                store_state<S>(dst + j * p.dstride + off, v.x, sizeof(S) == 2 ? rnd.template bits<j>() : 0u);
+                store_state<S>(dst + (Q - 1 - j) * p.dstride + off, v.y, sizeof(S) == 2 ? rnd.template bits<Q - 1 - j>() : 0u);
             });
             float ur;
             if constexpr (K::U0) {
@@ -1121,7 +1122,7 @@ __global__ void __launch_bounds__(512, 1)
                 const float f = cur[P::REST];
                 ur = fmaf(1.0f / 3.0f, f - (float)Store<S>::ld(src + NP * p.dstride + off), f);
             }
-            store_state_one<S>(dst + NP * p.dstride + off, ur, sizeof(S) == 2 ? rnd.template word<NP>() : 0u);
+            store_state<S>(dst + NP * p.dstride + off, ur, sizeof(S) == 2 ? rnd.template bits<NP>() : 0u);
         }
 #pragma unroll
         for (int i = 0; i < 4; i++) { Mx[i] = Mxn[i]; My[i] = Myn[i]; }
