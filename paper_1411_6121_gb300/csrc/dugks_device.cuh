@@ -318,6 +318,7 @@ struct StepParams {
 
 // Fills the FP32 copies above from the FP64 fields (host).
 inline void finish_step_params(StepParams &p) {
+    if (p.omega == 0.0) p.omega = 0.0;  // -0.0 has other bits: time_factors looks at the bits, the host at the value
     for (int w = 0; w < 6; w++) {
         for (int a = 0; a < 3; a++) {
             p.fwm[w][a] = (float)(p.bc_u[w][a] * p.rho0 * p.inv_c);
