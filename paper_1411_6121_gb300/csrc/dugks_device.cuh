@@ -112,21 +112,56 @@ __host__ __device__ constexpr int flux_index(int d, int k) {
 // ---------------------------------------------------------------------------------
 // Storage types
 // ---------------------------------------------------------------------------------
+// Loads of what the step before may still be writing while this grid is set up (launch_chained). The
+// non-coherent path (__ldg) wants memory that nobody writes during the grid's life; these are ordinary
+// loads, and volatile, so that none is moved above chain_wait().
+__device__ __forceinline__ float ld_chained(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_chained(const float2 *p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_chained(const double *p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_chained(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned short ld_chained(const unsigned short *p) {
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
+// ldc: the same value as ld, for the kernels of a chain (ld_chained).
 template <class S>
 struct Store;
 template <>
 struct Store<float> {
     __device__ static __forceinline__ float ld(const float *p) { return __ldg(p); }
+    __device__ static __forceinline__ float ldc(const float *p) { return ld_chained(p); }
     __device__ static __forceinline__ void st(float *p, float v) { *p = v; }
 };
 template <>
 struct Store<__nv_bfloat16> {
     __device__ static __forceinline__ float ld(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
+    __device__ static __forceinline__ float ldc(const __nv_bfloat16 *p) {
+        return __bfloat162float(__ushort_as_bfloat16(ld_chained(reinterpret_cast<const unsigned short *>(p))));
+    }
     __device__ static __forceinline__ void st(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 };
 template <>
 struct Store<double> {
     __device__ static __forceinline__ double ld(const double *p) { return __ldg(p); }
+    __device__ static __forceinline__ double ldc(const double *p) { return ld_chained(p); }
     __device__ static __forceinline__ void st(double *p, double v) { *p = v; }
 };
 // FP16 holds g~ * 2^12: the exact power-of-two scale moves FP16's normal range
@@ -136,6 +171,9 @@ constexpr float F16_SCALE = 4096.0f, F16_UNSCALE = 1.0f / 4096.0f;
 template <>
 struct Store<__half> {
     __device__ static __forceinline__ float ld(const __half *p) { return __half2float(__ldg(p)) * F16_UNSCALE; }
+    __device__ static __forceinline__ float ldc(const __half *p) {
+        return __half2float(__ushort_as_half(ld_chained(reinterpret_cast<const unsigned short *>(p)))) * F16_UNSCALE;
+    }
     __device__ static __forceinline__ void st(__half *p, float v) { *p = __float2half_rn(v * F16_SCALE); }
 };
 
@@ -229,7 +267,7 @@ __device__ __forceinline__ void store_state_one(S *p0, float v0, uint32_t r) {
 
 // A kernel launched as a programmatic dependent (launch_chained) may start before the work ahead of
 // it in its stream has ended; every thread waits for that work here before it touches memory, and
-// then lets the next such kernel start (which waits in turn).
+// then lets the next such kernel start (which waits in turn). What a step writes is read by ld_chained.
 __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
@@ -356,8 +394,8 @@ __device__ __forceinline__ void time_factors(const StepParams &p, T &ct, T &cth,
         cwh = T(1);
     } else if (!EVAL || p.tfac) {
         const TimeFactors *f = p.tfac + p.step_off;
-        if constexpr (sizeof(T) == 4) { ct = __ldg(&f->fct); cth = __ldg(&f->fcth); cwh = __ldg(&f->fcwh); }
-        else { ct = __ldg(&f->ct); cth = __ldg(&f->cth); cwh = __ldg(&f->cwh); }
+        if constexpr (sizeof(T) == 4) { ct = ld_chained(&f->fct); cth = ld_chained(&f->fcth); cwh = ld_chained(&f->fcwh); }
+        else { ct = ld_chained(&f->ct); cth = ld_chained(&f->cth); cwh = ld_chained(&f->cwh); }
     } else if constexpr (EVAL) {
         const TimeFactors f = eval_time_factors(p.omega, p.dt, p.inv_c, (double)(*p.step_ctr) + (double)p.step_off);
         ct = (T)f.ct;

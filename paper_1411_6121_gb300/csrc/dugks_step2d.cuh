@@ -150,13 +150,13 @@ __device__ __forceinline__ void load_row(const StepParams &p, const Strip &s, in
     if (s.vec) {
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            if constexpr (sizeof(S) == 4) g[k] = __ldg(reinterpret_cast<const float2 *>(row + k * p.dstride + s.ca));
-            else g[k] = unpack2(__ldg(reinterpret_cast<const uint32_t *>(row + k * p.dstride + s.ca)));
+            if constexpr (sizeof(S) == 4) g[k] = ld_chained(reinterpret_cast<const float2 *>(row + k * p.dstride + s.ca));
+            else g[k] = unpack2(ld_chained(reinterpret_cast<const uint32_t *>(row + k * p.dstride + s.ca)));
         }
     } else {
 #pragma unroll
         for (int k = 0; k < 9; k++)
-            g[k] = make_float2(Store<S>::ld(row + k * p.dstride + s.ca), Store<S>::ld(row + k * p.dstride + s.cb));
+            g[k] = make_float2(Store<S>::ldc(row + k * p.dstride + s.ca), Store<S>::ldc(row + k * p.dstride + s.cb));
     }
 }
 

@@ -213,7 +213,7 @@ __device__ __forceinline__ void step2d_tile(const StepParams &p, unsigned char *
         if (load) {
             const int64_t off = (int64_t)cy * p.px + cx;
 #pragma unroll
-            for (int k = 0; k < Q; k++) g[k] = (float)Store<S>::ld(src + k * p.dstride + off);
+            for (int k = 0; k < Q; k++) g[k] = (float)Store<S>::ldc(src + k * p.dstride + off);
             float Gh[3] = {0.0f, 0.0f, 0.0f}, drho, m[3];
             if (FORCE) cell_G<2, float>(p, (int64_t)cx + (int64_t)nx * cy, ncell, ct, Gh);
             moments<Q, float, true>(g, Gh, cf.wcell * cf.rho0, drho, m);

@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(32 * MAX_RY) fused_step2d_lean(const __grid_co
             T g[9], Gh[3] = {T(0), T(0), T(0)}, drho, mm[3];
             const int64_t off = (int64_t)cy * p.px + cx;
 #pragma unroll
-            for (int k = 0; k < 9; k++) g[k] = (T)Store<S>::ld(src + k * p.dstride + off);
+            for (int k = 0; k < 9; k++) g[k] = (T)Store<S>::ldc(src + k * p.dstride + off);
             if constexpr (FORCE) {
                 const int64_t c = (int64_t)cx + (int64_t)nx * cy;
                 if (p.field) {

@@ -1,5 +1,6 @@
 """The host side of a step's parameters, compiled and run without a GPU."""
 import os
+import re
 import subprocess
 
 import pytest
@@ -45,3 +46,24 @@ def test_kernels_and_host_agree_on_a_zero_omega(lines):
     """A kernel tells a steady force by the bits of omega, the host by its value: -0.0 must not reach the
     kernel, which would read a table that the host did not make."""
     assert lines == ["0 0", "0 0", "1 1", "1 1", "1 1"]
+
+
+def test_chained_kernels_read_states_by_coherent_loads():
+    """A kernel launched as a programmatic dependent is resident while the step before it still writes
+    the state: none may read the state, or the table of time factors, by the non-coherent path, which
+    wants memory that is read-only for the life of the grid."""
+    def code(name):
+        with open(os.path.join(_build.CSRC, name)) as f:
+            return re.sub(r"//[^\n]*", "", f.read())
+
+    chained = [n for n in sorted(os.listdir(_build.CSRC)) if n.endswith(".cuh") and "chain_wait();" in code(n)]
+    assert len(chained) >= 3
+    for name in chained:
+        text = code(name)
+        assert "Store<S>::ld(" not in text, name
+        for line in text.split("\n"):
+            for arg in re.findall(r"__ldg\(([^;]*)", line):  # what no step writes
+                assert re.match(r"(p\.field|p\.metric|fr \+|items)", arg), (name, line)
+    table = code("dugks_device.cuh")
+    table = table[table.index("void time_factors("):table.index("struct FromTable")]
+    assert "__ldg" not in table
