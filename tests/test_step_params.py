@@ -57,7 +57,7 @@ def test_chained_kernels_read_states_by_coherent_loads():
             return re.sub(r"//[^\n]*", "", f.read())
 
     chained = [n for n in sorted(os.listdir(_build.CSRC)) if n.endswith(".cuh") and "chain_wait();" in code(n)]
-    assert len(chained) >= 3
+    assert chained
     for name in chained:
         text = code(name)
         assert "Store<S>::ld(" not in text, name
