@@ -43,10 +43,14 @@
 // back (setmaxnreg to PROD_REGS) and the consumer warpgroups take them (CONS_REGS): 256 x 72 +
 // 256 x 184 = 512 x 128. Every wait on an mbarrier gives up after about two seconds (a device
 // flag, then the group leaves together; see tma.cuh).
-// Measured (ms per step, the non-specialised kernel / this one): 256^3 cavity 3.81 / 2.62, forced 157 x 101 x
-// 83 0.545 / 0.367. Written for any velocity set, and faster for D3Q19 as well (256^3 1.49 / 1.32), but D3Q19 keeps
-// dugks_step3d_ws.cuh: a steady flow, where every step rounds the same way, drifts from FP64 1.7
-// times as far there (32^3 cavity, 10,000 steps: 2.4e-6 against 1.4e-6).
+// The update adds the flux in increment form, La + b7 (W N' - La), with the weight W in head and tail: with
+// rounded (1 - b7) and b7 W, whose errors repeat at every step, forced and channel flows were up to 1.6 times
+// as far from FP64 as the non-specialised kernel after 20 steps. Error of the state / of u against FP64, this
+// kernel over the non-specialised one, geometric means over 36 random meshes (8 to 40 cells a side; channels on
+// three axes, forced, cavity, duct, periodic): 20 steps 0.86 / 0.92, 200 0.96 / 0.97, 1000 0.90 / 0.88, 4000 0.88 /
+// 0.88 (the worst family, cavities: 1.11 / 1.07 after 4000; the reference kernel scatters by 0.94 to 1.03).
+// Measured (ms, the non-specialised kernel / this one): a step of the 256^3 cavity 3.81 / 2.62; 20 steps of a
+// 157 x 101 x 83 channel under a force field, its moments and state read 13.9 / 8.3.
 #pragma once
 
 #include <math.h>
@@ -1036,7 +1040,7 @@ __global__ void __launch_bounds__(512, 1)
                     e2[i] = 3.0f * (D[a][1 + b] + D[b][1 + a]);
                 });
             }
-            const float tk = -cf.two_kappa * (FORCE ? 1.0f : cf.b7), lk = -cf.two_kappa * (1.0f - cf.b7);
+            const float mk = -cf.two_kappa, b7 = cf.b7;
             const int us = (nidx(kz) % 3) * K::NUC + (row - 1) * 32 + lane;
             const float *u0 = u0b + us * K::UP;
             const int64_t off = (int64_t)kz * p.plane + (int64_t)gy * p.px + gx;
@@ -1072,7 +1076,8 @@ __global__ void __launch_bounds__(512, 1)
                     }
                 }
                 La[j] = ln;
-                constexpr float w = Lat<Q>::w(j);
+                constexpr double W = Lat<Q>::template wt<double>(j);
+                constexpr float wh = (float)W, wl = (float)(W - (double)wh);
                 float2 n;
                 if constexpr (FORCE) {
                     n = N[j];
@@ -1108,8 +1113,16 @@ __global__ void __launch_bounds__(512, 1)
                     }
                     n = f2(E + O, E - O);
                 }
-                // eq. (16): f~(t+dt) = f~+ - dt/|V| flux
-                const float2 v = __fadd2_rn(u, __ffma2_rn(f2(tk * w, tk * w), n, __fmul2_rn(f2(lk, lk), l)));
+                // eq. (16): f~(t+dt) = f~+ - dt/|V| flux, the flux in increment form, La + b7 (W N' - La) (with
+                // a force N = b7 N'), with the weight in head and tail: see the header
+                float2 v;
+                if constexpr (FORCE) {
+                    const float2 t = __ffma2_rn(f2(wh, wh), n, __ffma2_rn(f2(wl, wl), n, __fmul2_rn(f2(-b7, -b7), l)));
+                    v = __ffma2_rn(f2(mk, mk), __fadd2_rn(l, t), u);
+                } else {
+                    const float2 t = __ffma2_rn(f2(wh, wh), n, sub2(__fmul2_rn(f2(wl, wl), n), l));
+                    v = __ffma2_rn(f2(mk, mk), __ffma2_rn(f2(b7, b7), t, l), u);
+                }
                 // the random bits that each value has in every kernel of the set
                 store_state<S>(dst + j * p.dstride + off, v.x, sizeof(S) == 2 ? rnd.template bits<j>() : 0u);
                 store_state<S>(dst + (Q - 1 - j) * p.dstride + off, v.y, sizeof(S) == 2 ? rnd.template bits<Q - 1 - j>() : 0u);
