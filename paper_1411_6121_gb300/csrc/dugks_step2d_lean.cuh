@@ -132,7 +132,8 @@ __global__ void __launch_bounds__(32 * MAX_RY) fused_step2d_lean(const __grid_co
     chain_wait();
     const Coef<T> cf(p);
     const int lane = threadIdx.x, row = threadIdx.y, ry = blockDim.y;
-    const int nx = p.nx, ny = p.ny, x0 = blockIdx.x * TXI, y0 = blockIdx.y * (ry - 2);
+    const int nx = p.nx, ny = p.ny, strips = (nx + TXI - 1) / TXI;
+    const int x0 = (int)(blockIdx.x % (unsigned)strips) * TXI, y0 = (int)(blockIdx.x / (unsigned)strips) * (ry - 2);
     const int gx = x0 - 1 + lane, gy = y0 - 1 + row;
     const int64_t ncell = (int64_t)nx * ny;
     const bool perx = p.bc[0] == 0, pery = p.bc[2] == 0;

@@ -40,7 +40,8 @@ cudaError_t launch(const StepParams &p, cudaStream_t stream) {
         configured_dev = dev;
     }
     const int ry = block_rows(p.nx, p.ny, sms);
-    const dim3 grid((p.nx + lean::TXI - 1) / lean::TXI, (p.ny + ry - 3) / (ry - 2));
+    // all tiles along x: a grid's y extent (65,535) would end at 393,210 rows of cells
+    const dim3 grid((unsigned)((int64_t)((p.nx + lean::TXI - 1) / lean::TXI) * ((p.ny + ry - 3) / (ry - 2))));
     return launch_chained(lean::fused_step2d_lean<S, NU, FORCE>, grid, dim3(32, ry), lean::smem_bytes<T, FORCE>(ry), stream,
                           p);
 }

@@ -133,3 +133,18 @@ def test_batch_read_back_by_pieces(shapes):
         assert np.array_equal(b.moments(i), one.moments())
         one.close()
     b.close()
+
+
+@pytest.mark.parametrize("shape", [(2, 400001), (1970000, 2)])
+def test_d2q9_lean_long_meshes(shape):
+    """FP64 meshes longer than a grid's y extent of tiles, along either axis: the general kernel's step."""
+    from paper_1411_6121_gb300 import dugks
+    p, u = W.random_state_fields(shape, seed=5, u_amp=0.03, p_amp=1e-3)
+    outs = []
+    for kernel in (0, 1):
+        s = dugks.Sim(shape, q=9, nu=0.05, dt=0.5, bcs=W.all_periodic(), store=3, kernel=kernel)
+        s.init(p=p, u=u)
+        s.step(2)
+        outs.append(s.get_state())
+        s.close()
+    assert np.abs(outs[0] - outs[1]).max() < 1e-11 * np.abs(outs[1]).max()
