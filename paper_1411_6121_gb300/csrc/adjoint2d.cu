@@ -539,6 +539,12 @@ __device__ __noinline__ void faces_frame_item(const AdjParams<T> &a, unsigned t)
     store(face_at(pos), Fb, Gb[0], Gb[1]);
 }
 
+// The frame item of a thread: eight per block of 128 threads, one per half-warp. From the block's number,
+// not the thread's: 16 threads an item pass 32 bits at 2^28 items (a long strip of 10^8 cells is all frame).
+__host__ __device__ constexpr unsigned frame_item(unsigned block, unsigned thread) { return block * 8u + (thread >> 4); }
+static_assert(frame_item(0, 127) == 7 && frame_item(1u << 25, 0) == 1u << 28 && frame_item((1u << 28) - 1, 127) == (1u << 31) - 1,
+              "frame items up to 2^31 - 1 have blocks and threads of their own");
+
 // Every interface of both axes in one launch of 128-thread blocks: the frame blocks first
 // (eight frame interfaces per block, one per half-warp), then 32 x 4 tiles of the interior
 // rectangle of x interfaces (nt0 tiles, tx0 per row), then those of y interfaces (tx1 per row).
@@ -546,7 +552,7 @@ template <class T>
 __global__ void __launch_bounds__(128, 6) adj_faces_all(const AdjParams<T> a, int64_t nframe, int nfb, int nt0,
                                                          int tx0, int tx1) {
     if ((int)blockIdx.x < nfb) {
-        const unsigned t = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+        const unsigned t = frame_item(blockIdx.x, threadIdx.x);
         if (t < nframe) faces_frame_item(a, t);
         return;
     }
@@ -664,7 +670,7 @@ template <class T>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 7 : 5) adj_cells_all(const AdjParams<T> a, int nfb, int tx, int ty) {
     const Rect r = cell_rect(a.n[0], a.n[1], a.per[0], a.per[1]);
     if ((int)blockIdx.x < nfb) {  // eight frame cells per block, one per half-warp
-        const unsigned t = blockIdx.x * 8 + (threadIdx.x >> 4);
+        const unsigned t = frame_item(blockIdx.x, threadIdx.x);
         if (t < frame_count(r)) cells_frame_item(a, t);
     } else {
         const int b = blockIdx.x - nfb;
