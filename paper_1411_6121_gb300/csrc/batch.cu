@@ -42,7 +42,8 @@ struct dugks_batch_s {
     int4 *d_items = nullptr;
     int nitems = 0, items_cap = 0;
     long long *d_step = nullptr;
-    float *d_mom = nullptr;  // staging of dugks_batch_moments to host memory (allocated on first use):
+    std::mutex staging;      // one host read-back of moments at a time: they share
+    float *d_mom = nullptr;  // the staging of dugks_batch_moments to host memory (allocated on first use):
     char *h_mom = nullptr;   // the largest instance's moments, and two page-locked pieces of MOM_PIECE bytes
     cudaEvent_t landed[2] = {nullptr, nullptr};
     int64_t step = 0;
@@ -435,7 +436,9 @@ int dugks_batch_moments(dugks_batch_t b, int32_t i, float *out, int32_t out_is_d
     const dugks_mesh &m = b->mesh[i];
     const size_t bytes = sizeof(float) * 3 * m.nx * m.ny;
     float *d = out;
+    std::unique_lock<std::mutex> one(b->staging, std::defer_lock);
     if (!out_is_device) {
+        one.lock();  // until the copy out has ended
         // staging of the largest instance, kept: an allocation and a release per call (each of which
         // waits for the device) took 0.2 ms of every host read-back
         if (!b->d_mom) {
