@@ -467,7 +467,7 @@ int dugks_moments(dugks_t h, float *out, int32_t out_is_device) {
 int dugks_residual(dugks_t h, double *out) {
     if (!h || !out) return DUGKS_E_INVAL;
     StepParams p = handle_params(h);
-    cudaError_t e = launch_residual(h->q, h->store, p, h->step * h->dt, h->rt, h->d_uprev, true, h->have_prev,
+    cudaError_t e = launch_residual(h->q, h->store, p, h->step * h->dt, h->rt, h->d_uprev, h->have_prev,
                                     h->d_partials, h->res_blocks, h->d_res, h->stream);
     h->launches += 2;
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_res, h->d_res, sizeof(double) * 8, cudaMemcpyDeviceToHost, h->stream);

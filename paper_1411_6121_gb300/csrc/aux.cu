@@ -1,6 +1,6 @@
 // aux.cu -- initialisation, moments and FP64 reductions of the DUGKS state (sm_103a).
 // The per-cell sums of 32- and 16-bit states run in FP32 as unevaluated pairs; the reductions
-// (residual, conservation totals) accumulate such pairs per thread and FP64 beyond.
+// (residual, conservation totals) go on in FP64.
 #include "dugks_internal.h"
 
 namespace dugks {
@@ -119,62 +119,59 @@ __device__ __forceinline__ Two<V> two_sum(V a, V b) {
     const V s = vadd(a, b), bb = vsub(s, a);
     return Two<V>{s, vadd(vsub(a, vsub(s, bb)), vsub(b, bb))};
 }
-// a + b of two such sums, to about 2^-47 of the larger.
-template <class V>
-__device__ __forceinline__ Two<V> two_add(Two<V> a, Two<V> b) {
-    const Two<V> t = two_sum(a.hi, b.hi);
-    return two_sum(t.hi, vadd(t.lo, vadd(a.lo, b.lo)));
-}
-// a b.
-template <class V>
-__device__ __forceinline__ Two<V> two_mul(Two<V> a, Two<V> b) {
-    const V p = vmul(a.hi, b.hi);
-    V e = vfma(a.hi, b.hi, vneg(p));
-    e = vfma(a.hi, b.lo, e);
-    e = vfma(a.lo, b.hi, e);
-    const V h = vadd(p, e);
-    return Two<V>{h, vsub(e, vsub(h, p))};
-}
-template <class V>
-__device__ __forceinline__ Two<V> two_set(double x) {
-    const float h = (float)x;
-    return Two<V>{vset(V(), h), vset(V(), (float)(x - (double)h))};
-}
-
 // Cell sums of a 32- or 16-bit state in FP32, each as an unevaluated pair: r = sum_k g_k and
-// j[a] = sum_k e_ka g_k. Every g_k is split into a head on the grid of 2^(E-16), where 2^E
-// bounds the cell's largest |g_k|, and a tail (adding and subtracting 1.5 * 2^(E+7)): the sums of
-// heads are exact (at most 27 terms below 2^(E+1)), and so are those of tails unless some
-// |g_k| is below 2^-13 of the largest, where they round near 2^(E-40). GB300 runs FP64 at a
-// 64th of its FP32 rate, so sums in FP64 would bound these kernels; TwoSum chains, which hold the
-// same, took 340 dependent operations per D3Q19 cell against about 140 for the split.
-template <int Q, class S, class V>
-__device__ __forceinline__ void cell_sums(const StepParams &p, const S *src, int64_t off, Two<V> &r, Two<V> j[3]) {
+// j[a] = sum_k e_ka g_k. With 2^E <= max |g_k| < 2^(E+1) every g_k is cut into a head on the grid of 2^(E-16)
+// (adding and subtracting 1.5 * 2^(E+7)), a middle part on that of 2^(E-33) and a tail: the sums of heads and of
+// middle parts are exact (at most 27 terms below 2^(E+1) and 2^(E-17)), the tails' round below 2^(E-50), and
+// head + middle is exact as a pair, whose low half takes the tail: 2^-48 of the sum itself. (Compensated
+// summation with TwoSum held 2^-48 of sum |g|, in 340 dependent operations per D3Q19 cell; with heads and
+// tails only, cells whose large values cancel lost 2^-41.) GB300 runs FP64 at a 64th of its FP32 rate, so
+// sums in FP64 would bound these kernels.
+template <class V>
+struct Three {
+    V h, m, t;
+    __device__ __forceinline__ void zero() { h = m = t = vset(V(), 0.0f); }
+    __device__ __forceinline__ void add(const Three &b) { h = vadd(h, b.h); m = vadd(m, b.m); t = vadd(t, b.t); }
+    __device__ __forceinline__ void sub(const Three &b) { h = vsub(h, b.h); m = vsub(m, b.m); t = vsub(t, b.t); }
+    __device__ __forceinline__ Two<V> pair() const {
+        const Two<V> p = two_sum(h, m);
+        return Two<V>{p.hi, vadd(p.lo, t)};
+    }
+};
+template <int Q, class V>
+__device__ __forceinline__ void cell_sums(const V g[Q], Two<V> &r, Two<V> j[3]) {
     constexpr int D = Lat<Q>::D, C = (Q - 1) / 2;  // velocities k and Q - 1 - k are opposite, C is at rest
-    V g[Q];
+    V big = vset(V(), 0.0f);
 #pragma unroll
-    for (int k = 0; k < Q; k++) g[k] = load_cells<V, S>(src + k * p.dstride + off);
-    V m = vset(V(), 0.0f);
+    for (int k = 0; k < Q; k++) big = vmaxabs(big, g[k]);
+    const V sp = split_of(big), sn = vneg(sp), mp = vmul(sp, vset(V(), 0x1p-17f)), mn = vneg(mp);
+    auto cut = [&](V v) __attribute__((always_inline)) {
+        Three<V> c;
+        c.h = vadd(vadd(v, sp), sn);
+        const V l = vsub(v, c.h);
+        c.m = vadd(vadd(l, mp), mn);
+        c.t = vsub(l, c.m);
+        return c;
+    };
+    Three<V> R = cut(g[C]), J[3];
 #pragma unroll
-    for (int k = 0; k < Q; k++) m = vmaxabs(m, g[k]);
-    const V sp = split_of(m), sn = vneg(sp);
-    r.hi = vadd(vadd(g[C], sp), sn);
-    r.lo = vsub(g[C], r.hi);
-#pragma unroll
-    for (int a = 0; a < 3; a++) j[a].hi = j[a].lo = vset(V(), 0.0f);
+    for (int a = 0; a < 3; a++) J[a].zero();
 #pragma unroll
     for (int k = 0; k < C; k++) {
-        const V h0 = vadd(vadd(g[k], sp), sn), h1 = vadd(vadd(g[Q - 1 - k], sp), sn);
-        const V l0 = vsub(g[k], h0), l1 = vsub(g[Q - 1 - k], h1);
-        r.hi = vadd(r.hi, vadd(h0, h1));
-        r.lo = vadd(r.lo, vadd(l0, l1));
-        const V dh = vsub(h0, h1), dl = vsub(l0, l1);
+        const Three<V> p = cut(g[k]), n = cut(g[Q - 1 - k]);
+        Three<V> s = p, d = p;
+        s.add(n);
+        d.sub(n);
+        R.add(s);
 #pragma unroll
         for (int a = 0; a < D; a++) {
-            if (Lat<Q>::e(k, a) > 0) { j[a].hi = vadd(j[a].hi, dh); j[a].lo = vadd(j[a].lo, dl); }
-            if (Lat<Q>::e(k, a) < 0) { j[a].hi = vsub(j[a].hi, dh); j[a].lo = vsub(j[a].lo, dl); }
+            if (Lat<Q>::e(k, a) > 0) J[a].add(d);
+            if (Lat<Q>::e(k, a) < 0) J[a].sub(d);
         }
     }
+    r = R.pair();
+#pragma unroll
+    for (int a = 0; a < D; a++) j[a] = J[a].pair();
 }
 
 // Element offset of cell n (x fastest) in the padded state layout: n itself when the rows carry
@@ -204,8 +201,12 @@ template <int Q, class S, class V>
 __device__ __forceinline__ void cell_moments_out_f(const StepParams &p, const S *src, int64_t n, int64_t ncell,
                                                    float ctdt, float c_over_rho0, float rt, float *out) {
     constexpr int D = Lat<Q>::D;
+    V g[Q];
+    const int64_t off = cell_offset(p, n, ncell);
+#pragma unroll
+    for (int k = 0; k < Q; k++) g[k] = load_cells<V, S>(src + k * p.dstride + off);
     Two<V> r, j[3];
-    cell_sums<Q, S, V>(p, src, cell_offset(p, n, ncell), r, j);
+    cell_sums<Q, V>(g, r, j);
     const V dr = vadd(r.hi, r.lo);
     store_out(out + n, vmul(dr, vset(V(), rt)));
     // c / rho0, or c / rho in the original model
@@ -221,7 +222,7 @@ __device__ __forceinline__ void cell_moments_out_f(const StepParams &p, const S 
 
 // Moments (eq. (27)): out[0] = p = (rho - rho0) RT, out[1+a] = u_a; [dim+1][ncell]. A pass over
 // the state bound by its bytes: V = float2 takes two cells per thread (64-bit loads, packed
-// arithmetic). 256^3 D3Q19 FP32, 1.54 GB: 536 us before, 268 us now (5.7 TB/s).
+// arithmetic). 256^3 D3Q19 FP32, 1.54 GB: 536 us before, 294 us now (5.2 TB/s).
 template <int Q, class S, class V>
 __global__ void __launch_bounds__(256) moments_kernel(const StepParams p, double ct, double rt, double c, float *out) {
     constexpr int D = Lat<Q>::D, NV = sizeof(V) / 4;
@@ -265,7 +266,26 @@ __device__ __forceinline__ void block_partials(const double s[RES_SLOTS], double
     }
 }
 
-// FP64 states, and the original model (whose velocity divides by the local density).
+// FP32 values as doubles by integer operations: a conversion takes the FP64 unit, at a 64th of the FP32 rate.
+// Not for subnormal, infinite and NaN values (odd_value).
+__device__ __forceinline__ bool odd_value(float x) {
+    const uint32_t m = __float_as_uint(x) & 0x7fffffffu;
+    return m - 0x00800000u >= 0x7f000000u && m != 0;
+}
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu, h = m != 0 ? (m >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)((b & 0x80000000u) | h), (int)(b << 29));
+}
+template <bool ODD>
+__device__ __forceinline__ double2 widen(Two<float2> v) {
+    if constexpr (ODD) return make_double2((double)v.hi.x + (double)v.lo.x, (double)v.hi.y + (double)v.lo.y);
+    else return make_double2(widen(v.hi.x) + widen(v.lo.x), widen(v.hi.y) + widen(v.lo.y));
+}
+__device__ __forceinline__ bool odd_value(Two<float2> v) {
+    return odd_value(v.hi.x) || odd_value(v.hi.y) || odd_value(v.lo.x) || odd_value(v.lo.y);
+}
+
+// FP64 states.
 template <int Q, class S>
 __global__ void __launch_bounds__(RES_THREADS) residual_kernel(const StepParams p, double ct, double c, double *uprev,
                                                                 int have_prev, double *partials) {
@@ -288,81 +308,102 @@ __global__ void __launch_bounds__(RES_THREADS) residual_kernel(const StepParams 
     block_partials(s, partials);
 }
 
-// 32- and 16-bit states of the incompressible model. Each cell's velocity u / c = sum e g / rho0 +
-// shift is formed, differenced, squared and summed over the thread's cells as an unevaluated
-// pair of FP32 values (about 47 bits; the squares are taken of 2^30 u / c, which keeps the low
-// parts of slow flows in range), and goes to FP64 once per thread: a pass over the state bound
-// by its bytes instead of 37 FP64 instructions per cell at a 64th of the FP32 rate. PAIR: u_prev
-// is the handle's own and holds those pairs; otherwise it is the caller's array of doubles.
-// 256^3 D3Q19 FP32, 2.08 GB: 2626 us before, 316 us now (6.6 TB/s).
-constexpr float SQ_SCALE = 1073741824.0f;  // 2^30
-// u_prev / c of V's cells (zero before any).
-template <class V, bool PAIR>
-__device__ __forceinline__ Two<V> load_prev(const double *up, int have_prev, double c) {
-    static_assert(PAIR || sizeof(V) == 4, "the caller's array is taken one cell at a time");
-    Two<V> r = {vset(V(), 0.0f), vset(V(), 0.0f)};
-    if (!have_prev) return r;
-    if constexpr (!PAIR) {
-        r = two_set<V>(*up / c);
-    } else if constexpr (sizeof(V) == 4) {
-        const float2 v = *reinterpret_cast<const float2 *>(up);
-        r = Two<V>{v.x, v.y};
-    } else {
-        const float4 v = *reinterpret_cast<const float4 *>(up);
-        r = Two<V>{make_float2(v.x, v.z), make_float2(v.y, v.w)};
-    }
-    return r;
-}
-template <int Q, class S, class V, bool PAIR>
+// 32- and 16-bit states: the cell sums in FP32 (cell_sums), then FP64 per cell: u, its difference, the squares
+// and the sums. A thread takes the cells n and n + 1, VEC: by loads of both at once; the order of the sums
+// is the same either way. ORIG: the original model, whose velocity divides by the local density.
+// 256^3 D3Q19 FP32, 2.08 GB (us): 2626 with one thread per cell, conversions and u_prev behind the stores,
+// 670 now: 21 FP64 instructions per cell, the FP64 unit 83% busy. (Pairs of floats all the way took 316, but
+// hold 47 bits and the range of FP32.)
+template <int Q, class S, bool VEC, bool ORIG>
 __global__ void __launch_bounds__(RES_THREADS) residual_kernel_f(const StepParams p, double ct, double c, double *uprev,
                                                                   int have_prev, double *partials) {
-    constexpr int D = Lat<Q>::D, NV = sizeof(V) / 4;
+    constexpr int D = Lat<Q>::D;
     const int64_t ncell = (int64_t)p.nx * p.ny * p.nz;
     const S *src = reinterpret_cast<const S *>(p.src);
-    const Two<V> zero = {vset(V(), 0.0f), vset(V(), 0.0f)};
-    const Two<V> ir = two_set<V>(1.0 / p.rho0), cs = two_set<V>(ct * 0.5 * p.dt / c);  // shift = (g + field) cs
-    Two<V> sh[3];
+    const double cr0 = c / p.rho0, dtc = 0.5 * p.dt;
+    double shift[3];
 #pragma unroll
-    for (int a = 0; a < 3; a++) sh[a] = two_set<V>(p.g[a] * (ct * 0.5 * p.dt / c));
-    const bool shifted = p.g[0] != 0.0 || p.g[1] != 0.0 || p.g[2] != 0.0;
-    Two<V> s0 = zero, s1 = zero, s2 = zero, su[3] = {zero, zero, zero};
+    for (int a = 0; a < 3; a++) shift[a] = p.g[a] * ct * dtc;
+    double s[RES_SLOTS] = {0, 0, 0, 0, 0, 0, 0, 0};
     int64_t cells = 0;
-    for (int64_t n = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * NV; n < ncell;
-         n += (int64_t)gridDim.x * blockDim.x * NV) {
+    for (int64_t n = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); n < ncell;
+         n += 2 * (int64_t)gridDim.x * blockDim.x) {
+        const int64_t n1 = VEC || n + 1 < ncell ? n + 1 : n;
         // u_prev first: its loads must not wait behind the stores of u below (which the compiler
         // has to order, axis by axis) or behind the sums
-        Two<V> before[3];
-#pragma unroll
-        for (int a = 0; a < D; a++) before[a] = load_prev<V, PAIR>(uprev + a * ncell + n, have_prev, c);
-        Two<V> r, j[3];
-        cell_sums<Q, S, V>(p, src, cell_offset(p, n, ncell), r, j);
-        s2 = two_add(s2, r);
-        cells += NV;
+        double2 before[3];
 #pragma unroll
         for (int a = 0; a < D; a++) {
-            Two<V> u = two_mul(two_sum(j[a].hi, j[a].lo), ir);
-            if (shifted) u = two_add(u, sh[a]);
-            if (p.field) u = two_add(u, two_mul(Two<V>{load_field(p.field + a * ncell + n, V()), zero.lo}, cs));
-            double *up = uprev + a * ncell + n;
-            if constexpr (!PAIR) *up = ((double)u.hi + (double)u.lo) * c;
-            else if constexpr (NV == 2) *reinterpret_cast<float4 *>(up) = make_float4(u.hi.x, u.lo.x, u.hi.y, u.lo.y);
-            else *reinterpret_cast<float2 *>(up) = make_float2(u.hi, u.lo);
-            Two<V> du = two_add(u, Two<V>{vneg(before[a].hi), vneg(before[a].lo)});
-            du = Two<V>{vmul(du.hi, vset(V(), SQ_SCALE)), vmul(du.lo, vset(V(), SQ_SCALE))};
-            const Two<V> us = {vmul(u.hi, vset(V(), SQ_SCALE)), vmul(u.lo, vset(V(), SQ_SCALE))};
-            s0 = two_add(s0, two_mul(du, du));
-            s1 = two_add(s1, two_mul(us, us));
-            su[a] = two_add(su[a], u);
+            const double *up = uprev + a * ncell;
+            if (!have_prev) before[a] = make_double2(0.0, 0.0);
+            else if constexpr (VEC) before[a] = *reinterpret_cast<const double2 *>(up + n);
+            else before[a] = make_double2(up[n], up[n1]);
+        }
+        float2 g[Q];
+        const int64_t off = cell_offset(p, n, ncell), off1 = VEC ? off : cell_offset(p, n1, ncell);
+#pragma unroll
+        for (int k = 0; k < Q; k++) {
+            const S *q = src + k * p.dstride;
+            if constexpr (VEC) g[k] = load_cells<float2, S>(q + off);
+            else g[k] = make_float2(Store<S>::ld(q + off), Store<S>::ld(q + off1));
+        }
+        Two<float2> r, j[3];
+        cell_sums<Q, float2>(g, r, j);
+        double2 u[3], drho;  // u: the momenta first
+        bool odd = odd_value(r);
+#pragma unroll
+        for (int a = 0; a < D; a++) odd = odd || odd_value(j[a]);
+        if (odd) {
+            drho = widen<true>(r);
+#pragma unroll
+            for (int a = 0; a < D; a++) u[a] = widen<true>(j[a]);
+        } else {
+            drho = widen<false>(r);
+#pragma unroll
+            for (int a = 0; a < D; a++) u[a] = widen<false>(j[a]);
+        }
+        double2 cr = make_double2(cr0, cr0);
+        if constexpr (ORIG) cr = make_double2(c / (p.rho0 + drho.x), c / (p.rho0 + drho.y));
+        double2 sh[3];
+#pragma unroll
+        for (int a = 0; a < D; a++) sh[a] = make_double2(shift[a], shift[a]);
+        if (p.field) {  // one block of all axes: a real branch, not predicated FP64 operations
+#pragma unroll
+            for (int a = 0; a < D; a++) {
+                const float *f = p.field + a * ncell;
+                sh[a] = make_double2((p.g[a] + (double)__ldg(f + n)) * ct * dtc, (p.g[a] + (double)__ldg(f + n1)) * ct * dtc);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < D; a++) {
+            u[a] = make_double2(fma(cr.x, u[a].x, sh[a].x), fma(cr.y, u[a].y, sh[a].y));
+            double *up = uprev + a * ncell;
+            if constexpr (VEC) *reinterpret_cast<double2 *>(up + n) = u[a];
+            else {
+                up[n] = u[a].x;
+                if (n1 != n) up[n1] = u[a].y;
+            }
+        }
+        auto take = [&](double dr, const double v[3], const double b[3]) __attribute__((always_inline)) {
+            const double rho = ORIG ? p.rho0 + dr : p.rho0;
+#pragma unroll
+            for (int a = 0; a < D; a++) {
+                const double du = v[a] - b[a];
+                s[0] = fma(du, du, s[0]);
+                s[1] = fma(v[a], v[a], s[1]);
+                s[3 + a] = fma(rho, v[a], s[3 + a]);  // rho0 u, or rho u
+            }
+            s[2] += dr;
+            cells++;
+        };
+        const double ux[3] = {u[0].x, u[1].x, D == 3 ? u[2].x : 0.0}, bx[3] = {before[0].x, before[1].x, D == 3 ? before[2].x : 0.0};
+        take(drho.x, ux, bx);
+        if (n1 != n) {
+            const double uy[3] = {u[0].y, u[1].y, D == 3 ? u[2].y : 0.0}, by[3] = {before[0].y, before[1].y, D == 3 ? before[2].y : 0.0};
+            take(drho.y, uy, by);
         }
     }
-    auto total = [](const Two<V> &t) -> double {
-        if constexpr (NV == 2) return ((double)t.hi.x + (double)t.lo.x) + ((double)t.hi.y + (double)t.lo.y);
-        else return (double)t.hi + (double)t.lo;
-    };
-    const double q2 = (c / SQ_SCALE) * (c / SQ_SCALE);
-    double s[RES_SLOTS] = {total(s0) * q2, total(s1) * q2, p.rho0 * (double)cells + total(s2), 0, 0, 0, 0, 0};
-#pragma unroll
-    for (int a = 0; a < D; a++) s[3 + a] = p.rho0 * c * total(su[a]);
+    s[2] = fma(p.rho0, (double)cells, s[2]);
     block_partials(s, partials);
 }
 
@@ -437,30 +478,30 @@ static cudaError_t moments_q(int store, const StepParams &p, double t, double rt
     return cudaGetLastError();
 }
 
-template <int Q, class S>
-static void residual_s(const StepParams &p, int store, double ct, double c, double *uprev, bool pair, int have_prev,
-                       double *partials, int nblocks, cudaStream_t st) {
-    if (!pair) residual_kernel_f<Q, S, float, false><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
-    else if (pairs_ok(p, store, uprev, 16))
-        residual_kernel_f<Q, S, float2, true><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
+template <int Q, class S, bool ORIG>
+static void residual_m(const StepParams &p, int store, double ct, double c, double *uprev, int have_prev, double *partials,
+                       int nblocks, cudaStream_t st) {
+    if (pairs_ok(p, store, uprev, 16))
+        residual_kernel_f<Q, S, true, ORIG><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
     else
-        residual_kernel_f<Q, S, float, true><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
+        residual_kernel_f<Q, S, false, ORIG><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
+}
+
+template <int Q, class S>
+static void residual_s(const StepParams &p, int store, double ct, double c, double *uprev, int have_prev, double *partials,
+                       int nblocks, cudaStream_t st) {
+    if (p.model == 1) residual_m<Q, S, true>(p, store, ct, c, uprev, have_prev, partials, nblocks, st);
+    else residual_m<Q, S, false>(p, store, ct, c, uprev, have_prev, partials, nblocks, st);
 }
 
 template <int Q>
-static cudaError_t residual_q(int store, const StepParams &p, double t, double rt, double *uprev, bool pair,
-                              int have_prev, double *partials, int nblocks, double *out, cudaStream_t st) {
+static cudaError_t residual_q(int store, const StepParams &p, double t, double rt, double *uprev, int have_prev,
+                              double *partials, int nblocks, double *out, cudaStream_t st) {
     const double c = sqrt(3.0 * rt);
     const double ct = cos(p.omega * t);
-    const bool orig = p.model == 1;
-    if (store == 0 && !orig) residual_s<Q, float>(p, store, ct, c, uprev, pair, have_prev, partials, nblocks, st);
-    else if (store == 1 && !orig)
-        residual_s<Q, __nv_bfloat16>(p, store, ct, c, uprev, pair, have_prev, partials, nblocks, st);
-    else if (store == 2 && !orig) residual_s<Q, __half>(p, store, ct, c, uprev, pair, have_prev, partials, nblocks, st);
-    else if (store == 0) residual_kernel<Q, float><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
-    else if (store == 1)
-        residual_kernel<Q, __nv_bfloat16><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
-    else if (store == 2) residual_kernel<Q, __half><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
+    if (store == 0) residual_s<Q, float>(p, store, ct, c, uprev, have_prev, partials, nblocks, st);
+    else if (store == 1) residual_s<Q, __nv_bfloat16>(p, store, ct, c, uprev, have_prev, partials, nblocks, st);
+    else if (store == 2) residual_s<Q, __half>(p, store, ct, c, uprev, have_prev, partials, nblocks, st);
     else residual_kernel<Q, double><<<nblocks, RES_THREADS, 0, st>>>(p, ct, c, uprev, have_prev, partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -487,12 +528,12 @@ cudaError_t launch_moments(int q, int store, const StepParams &p, double t, doub
     return cudaErrorNotSupported;
 }
 
-cudaError_t launch_residual(int q, int store, const StepParams &p, double t, double rt, double *uprev, bool pair,
+cudaError_t launch_residual(int q, int store, const StepParams &p, double t, double rt, double *uprev,
                             int have_prev, double *partials, int nblocks, double *out, cudaStream_t st) {
     switch (q) {
-        case 9: return residual_q<9>(store, p, t, rt, uprev, pair, have_prev, partials, nblocks, out, st);
-        case 19: return residual_q<19>(store, p, t, rt, uprev, pair, have_prev, partials, nblocks, out, st);
-        case 27: return residual_q<27>(store, p, t, rt, uprev, pair, have_prev, partials, nblocks, out, st);
+        case 9: return residual_q<9>(store, p, t, rt, uprev, have_prev, partials, nblocks, out, st);
+        case 19: return residual_q<19>(store, p, t, rt, uprev, have_prev, partials, nblocks, out, st);
+        case 27: return residual_q<27>(store, p, t, rt, uprev, have_prev, partials, nblocks, out, st);
     }
     return cudaErrorNotSupported;
 }

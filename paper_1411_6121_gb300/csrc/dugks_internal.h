@@ -66,9 +66,8 @@ cudaError_t launch_moments(int q, int store, const StepParams &p, double t, doub
                            cudaStream_t stream);
 // FP64 residual and totals: per-block partial sums into `partials` ([nblocks][8] doubles),
 // then a fixed-order final sum into `out` (8 doubles on the device).
-// `pair`: uprev is the handle's own buffer, which holds the velocity / c of 32- and 16-bit states
-// (incompressible model) as pairs of floats; otherwise an array of doubles holding u.
-cudaError_t launch_residual(int q, int store, const StepParams &p, double t, double rt, double *uprev, bool pair,
+// uprev: [dim][ncell] u of the call before, overwritten.
+cudaError_t launch_residual(int q, int store, const StepParams &p, double t, double rt, double *uprev,
                             int have_prev, double *partials, int nblocks, double *out, cudaStream_t stream);
 int residual_blocks(int64_t ncell);
 // The time factors of the n steps from the device step counter on into out[0 .. n-1].

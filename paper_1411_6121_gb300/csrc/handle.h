@@ -67,7 +67,7 @@ struct dugks_s {
     long long *d_step;     // device step counter
     dugks::TimeFactors *d_tfac;  // [STEP_CHUNK] time factors of the steps being enqueued (omega != 0)
     int64_t step;          // host mirror of the step counter
-    double *d_uprev;       // [dim][ncell] velocity at the previous residual (format: launch_residual)
+    double *d_uprev;       // [dim][ncell] velocity at the previous residual
     int have_prev;
     double *d_partials;
     int res_blocks;

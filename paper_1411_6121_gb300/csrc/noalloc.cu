@@ -113,7 +113,7 @@ extern "C" int dugks_residual_static(int32_t lattice, int32_t store, const void 
     p.dt = 2.0;
     p.src = state;
     cudaStream_t st = (cudaStream_t)stream;
-    e = launch_residual(lattice, store, p, 0.0, rt, uprev, false, have_prev ? 1 : 0, partials, nblocks, final_sum, st);
+    e = launch_residual(lattice, store, p, 0.0, rt, uprev, have_prev ? 1 : 0, partials, nblocks, final_sum, st);
     double s[8];
     if (e == cudaSuccess) e = cudaMemcpyAsync(s, final_sum, sizeof s, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
