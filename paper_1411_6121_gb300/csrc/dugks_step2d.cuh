@@ -30,11 +30,11 @@
 //    equilibrium flux telescopes exactly.
 //  * At a wall interface step 5 replaces the incoming velocities' F: the interface moments get
 //    the sum of the changes, and the cell's La the changes themselves.
-//  * The update adds the flux in increment form, La + b7 (W N' - La), with the weights in head and tail:
-//    rounded (1 - b7) and b7 W would repeat their errors at every step. Error of the state / of u against
-//    FP64 over that of the one-cell kernel (dugks_step2d_cell.cuh), geometric means over 64 random meshes (8 to
-//    200 cells a side, six kinds of flow): 20 steps 0.92 / 0.91, 200 0.95 / 0.95, 1000 0.91 / 0.88. Cost: 0.5%
-//    of a 1024^2 step.
+//  * The update adds (1 - b7) La + b7 W N with both coefficients rounded on their own. Error of the state / of u
+//    against FP64 over that of the one-cell kernel (dugks_step2d_cell.cuh), geometric means over 64 random
+//    meshes (8 to 200 cells a side, six kinds of flow): 20 steps 0.94 / 0.93, 200 0.98 / 0.95, 1000 0.92 / 0.88. The
+//    increment form with split weights of dugks_step3d_ws27.cuh gave 0.92 / 0.91, 0.95 / 0.95, 0.91 / 0.88 for 1% of a
+//    batch's time.
 // Measured (us per step, one instance, before / now; before: one cell per thread, 32 x 8 threads, 30
 // warp instructions per cell, 56% issue): 1024^2 cavity 40.0 / 27.2 (16 instructions per cell, 53%
 // issue, 24 warps per SM), 2048^2 155 / 102, 512 x 256 channel 8.8 / 6.8, 8 x 32 channel 3.45 / 3.2 (the
@@ -756,24 +756,14 @@ __device__ __forceinline__ void tile(const StepParams &p, V *sm, int x0, int y0)
         N[6] = add(em, om);
         N[2] = sub(em, om);
     }
-    // ---- step 9, eq. (16), the flux in increment form, La + b7 (W N' - La) (with a force N = b7 N'), with
-    // the weights in head and tail (those of the diagonals a quarter: exact) ----
-    constexpr double W = 1.0 / 9.0;
-    constexpr float wh = (float)W, wl = (float)(W - (double)wh);
-    const V b7 = bc(FORCE ? -cf.b7 : cf.b7), mk = bc(-cf.two_kappa);
+    // ---- step 9, eq. (16) ----
+    const float tk = -cf.two_kappa * (FORCE ? 1.0f : cf.b7);
+    const V cL = bc(-cf.two_kappa * (1.0f - cf.b7)), w1 = bc(tk * (1.0f / 9.0f)), w2 = bc(tk * (1.0f / 36.0f));
     V u0[9];
 #pragma unroll
     for (int k = 0; k < 9; k++) {
         u0[k] = pub(0, PU + k);
-        if (k == 4) continue;
-        const float q = ex(k) != 0 && ey(k) != 0 ? 0.25f : 1.0f;
-        if constexpr (FORCE) {
-            const V t = fma(bc(q * wh), N[k], fma(bc(q * wl), N[k], mul(b7, La[k])));
-            u0[k] = fma(mk, add(La[k], t), u0[k]);
-        } else {
-            const V t = fma(bc(q * wh), N[k], sub(mul(bc(q * wl), N[k]), La[k]));
-            u0[k] = fma(mk, fma(b7, t, La[k]), u0[k]);
-        }
+        if (k != 4) u0[k] = add(u0[k], fma(ex(k) != 0 && ey(k) != 0 ? w2 : w1, N[k], mul(cL, La[k])));
     }
     const bool mine = s.lane >= 1 && s.lane <= TXI / 2;
     const bool upd0 = mine && s.gx0 < p.nx, upd1 = mine && s.gx0 + 1 < p.nx;
