@@ -63,15 +63,6 @@ constexpr int REG_THREADS = 768;
 
 using V = float2;
 __device__ __forceinline__ V bc(float x) { return make_float2(x, x); }
-__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-template <class T>
-__device__ __forceinline__ T all(float x) {
-    if constexpr (sizeof(T) == 4) return x;
-    else return make_float2(x, x);
-}
 __device__ __forceinline__ V add(V a, V b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ V mul(V a, V b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ V fma(V a, V b, V c) { return __ffma2_rn(a, b, c); }
@@ -340,55 +331,52 @@ __device__ __forceinline__ void face_numbers(const Coef<float> &cf, const V fm[3
 }
 
 // f_eq deviation of velocity k over the cells (geq_k).
-template <int k, class T>
-__device__ __forceinline__ T geq2(const Coef<float> &cf, T dr, T mx, T my) {
+template <int k>
+__device__ __forceinline__ V geq2(const Coef<float> &cf, V dr, V mx, V my) {
     const float ir = cf.inv_rho0;
-    const T mm = fma(mx, mx, mul(my, my));
-    T em = all<T>(0.0f);
+    const V mm = fma(mx, mx, mul(my, my));
+    V em = bc(0.0f);
     if (ex(k) > 0) em = mx;
-    if (ex(k) < 0) em = mul(all<T>(-1.0f), mx);
+    if (ex(k) < 0) em = mul(bc(-1.0f), mx);
     if (ey(k) > 0) em = ex(k) ? add(em, my) : my;
-    if (ey(k) < 0) em = ex(k) ? sub(em, my) : mul(all<T>(-1.0f), my);
-    const T x = fma(em, all<T>(3.0f), fma(mul(all<T>(ir), em), mul(all<T>(4.5f), em), fma(all<T>(-1.5f * ir), mm, dr)));
+    if (ey(k) < 0) em = ex(k) ? sub(em, my) : mul(bc(-1.0f), my);
+    const V x = fma(em, bc(3.0f), fma(mul(bc(ir), em), mul(bc(4.5f), em), fma(bc(-1.5f * ir), mm, dr)));
     constexpr double W = Lat<9>::wt<double>(k);
     constexpr float wh = (float)W, wl = (float)(W - (double)wh);
-    return fma(all<T>(wl), x, mul(all<T>(wh), x));
+    return fma(bc(wl), x, mul(bc(wh), x));
 }
 
-// Step 5 for the incoming velocities kin[0..2] (t component -1, 0, 1) of a wall normal to axis d:
-// their new values minus the step-4 ones. Fi, Fo: step-4 values of the incoming velocities and of
-// their opposites at the wall; Fc at x_c; cm: drho, j_n, j_t at x_c; Gc: acceleration / c there.
-// Adds the change to the wall's moments wm (drho, j_n, j_t).
-template <int d, int side, bool FORCE, class T>
-__device__ __forceinline__ void wall_change(const StepParams &p, const Coef<float> &cf, const T Fi[3], const T Fo[3],
-                                            const T Fc[3], const T cm[3], T Gcn, T Gct, T wm[3], T dF[3]) {
-    constexpr int wid = 2 * d + side, sg = side == 0 ? 1 : -1;  // sg: the incoming velocities' e_n
+// Step 5 for the incoming velocities (e_x -1, 0, 1) of a y wall: their new values minus the step-4 ones.
+// Fi, Fo: step-4 values of the incoming velocities and of their opposites at the wall; Fc at x_c; cm:
+// drho, j_y, j_x at x_c; Gcy, Gcx: acceleration / c there. Adds the change to the wall's moments wm
+// (drho, j_y, j_x).
+template <int side, bool FORCE>
+__device__ __forceinline__ void wall_change(const StepParams &p, const Coef<float> &cf, const V Fi[3], const V Fo[3],
+                                            const V Fc[3], const V cm[3], V Gcy, V Gcx, V wm[3], V dF[3]) {
+    constexpr int wid = 2 + side, sg = side == 0 ? 1 : -1;  // sg: the incoming velocities' e_y
     const float *mw = p.fwm[wid];
-    T mc[2] = {cm[1], cm[2]};  // normal, tangential
+    V my = cm[1], mx = cm[2];
     if constexpr (FORCE) {
-        const T w = all<T>(cf.wface * cf.rho0);
-        mc[0] = fma(Gcn, w, mc[0]);
-        mc[1] = fma(Gct, w, mc[1]);
+        const V w = bc(cf.wface * cf.rho0);
+        my = fma(Gcy, w, my);
+        mx = fma(Gcx, w, mx);
     }
     const int type = p.bc[wid];
     const bool vel = type == 1;
-    const T dra = vel ? cm[0] : all<T>(wall_drho<float>(p, cf, wid));
-    const T man = vel ? all<T>(mw[d]) : mc[0], mat = vel ? all<T>(mw[1 - d]) : mc[1];
+    const V dra = vel ? cm[0] : bc(wall_drho<float>(p, cf, wid));
+    const V m_ay = vel ? bc(mw[1]) : my, m_ax = vel ? bc(mw[0]) : mx;
     sfor<3>([&](auto ic) {
-        constexpr int i = ic, t = i - 1;
-        constexpr int k = d == 0 ? 3 * (sg + 1) + t + 1 : 3 * (t + 1) + sg + 1;
-        T v;
+        constexpr int i = ic, t = i - 1, k = 3 * (t + 1) + sg + 1;
+        V v;
         if (type == 3) {
-            const float em = (float)sg * mw[d] + (float)t * mw[1 - d];
-            v = add(Fo[i], all<T>(wmul<9, float>(k, 6.0f * em)));
+            const float em = (float)sg * mw[1] + (float)t * mw[0];
+            v = add(Fo[i], bc(wmul<9, float>(k, 6.0f * em)));
         } else {
-            const T a = d == 0 ? geq2<k>(cf, dra, man, mat) : geq2<k>(cf, dra, mat, man);
-            const T c = d == 0 ? geq2<k>(cf, cm[0], mc[0], mc[1]) : geq2<k>(cf, cm[0], mc[1], mc[0]);
-            v = add(a, sub(Fc[i], c));
+            v = add(geq2<k>(cf, dra, m_ax, m_ay), sub(Fc[i], geq2<k>(cf, cm[0], mx, my)));
         }
         dF[i] = sub(v, Fi[i]);
     });
-    const T s = add(add(dF[0], dF[1]), dF[2]);
+    const V s = add(add(dF[0], dF[1]), dF[2]);
     wm[0] = add(wm[0], s);
     wm[1] = sg > 0 ? add(wm[1], s) : sub(wm[1], s);
     wm[2] = add(wm[2], sub(dF[2], dF[0]));
@@ -425,7 +413,7 @@ __device__ __forceinline__ void y_wall(const StepParams &p, const Coef<float> &c
         for (int c = 0; c < 2; c++)
             Gc[c] = mul(add(bc(p.fg[c]), mul(bc(0.5f), add(pub(dc, PFLD + c), pub(dc + 1, PFLD + c)))), bc(cf.cth));
     }
-    wall_change<1, side, FORCE>(p, cf, Fi, Fo, Fc, cm, Gc[1], Gc[0], wm, dF);
+    wall_change<side, FORCE>(p, cf, Fi, Fo, Fc, cm, Gc[1], Gc[0], wm, dF);
 #pragma unroll
     for (int i = 0; i < 3; i++) {
         pub(0, PU + i) = wm[i];

@@ -807,4 +807,20 @@ __device__ __forceinline__ void step3d_segment(const StepParams &p, const CUtens
     }
 }
 
+// z chunk length for tiles of columns on `slots` resident CTAs: maximise (useful waves / launched waves) /
+// (1 + 2 / chunk length) (each chunk makes two extra planes of fbar+ in its prologue).
+inline int zchunk_for(int64_t tiles, int nz, int64_t slots) {
+    int best = 1;
+    double best_eff = -1.0;
+    for (int nc = 1; nc <= 16; nc++) {
+        const int zc = (nz + nc - 1) / nc;
+        if (nc > 1 && zc < 8) break;
+        const int ncr = (nz + zc - 1) / zc;
+        const double waves = (double)(tiles * ncr) / (double)slots;
+        const double eff = waves / ceil(waves) / (1.0 + 2.0 / zc);
+        if (eff > best_eff + 1e-9) { best_eff = eff; best = nc; }
+    }
+    return (nz + best - 1) / best;
+}
+
 }  // namespace dugks

@@ -4,12 +4,11 @@
 // and the arithmetic done on pairs of opposite velocities.
 //
 //  * Producer warps (8, one cell column each) make step 1: the state of the tile's plane arrives by
-//    TMA into one shared-memory stage, each column forms fbar+ and its moments (and, for D3Q19, u0 =
-//    g~ + 4/3 (fbar+ - g~) of the update), then the ghost columns and rows (step 2) and, beyond
-//    non-periodic z walls, the ghost planes.
+//    TMA into one shared-memory stage, each column forms fbar+ and its moments, then the ghost columns
+//    and rows (step 2) and, beyond non-periodic z walls, the ghost planes.
 //  * Consumer warps (8, one cell column each) do the rest for plane kz.
-//  * The planes pass through a ring of four slots (fbar+ and moments) and, for D3Q19, three u0 slots.
-//    Each ring slot has a "full" mbarrier (every producer thread arrives after its last write of the
+//  * The planes pass through a ring of four slots (fbar+ and moments). u0 = 4/3 fbar+ - 1/3 g~ of the update
+//    has no room beside them: the consumers read g~ a second time. Each ring slot has a "full" mbarrier (every producer thread arrives after its last write of the
 //    plane) and an "empty" one (every consumer thread arrives after its last read), so neither
 //    group waits on a CTA-wide barrier: the producer runs up to two planes ahead. The consumers'
 //    y exchange and the producers' ghost passes use named barriers of their own group.
@@ -23,14 +22,14 @@
 // is formed per pair of opposite velocities from differences of neighbouring cells, and
 // N = sum_d e_d [Y(+d) - Y(-d)]. No step-4 value is formed at an inner interface. Y needs only the
 // interface's moments, formed in moment space (A(L) + B(R), A, B = M/2 +- kappa M_d - kappa/4 dt M_t).
-// Without a force the brackets of all velocities that cross the interface are polynomials of 8
-// (D3Q19) or 10 (D3Q27) numbers, which are differenced across the cell and combined; with a force the
+// Without a force the brackets of all velocities that cross the interface are polynomials of
+// ten numbers, which are differenced across the cell and combined; with a force the
 // brackets themselves are. Both cells of an interface use the same numbers, so the equilibrium
 // flux telescopes exactly. The z march keeps La, the x and y differences and the numbers of the -z
 // interface in registers. At a wall interface: x, step 5 changes the interface's moments and La; y
 // and z, the direct path (all velocities) gives f there, and its numbers are zero.
 //
-// Pairs. Both velocity orders put opposite velocities at k and Q - 1 - k (the rest velocity in
+// Pairs. The velocity order puts opposite velocities at k and Q - 1 - k (the rest velocity in
 // the middle), so the moving velocities form pairs (j, Q - 1 - j) with e_{Q-1-j} = -e_j. Every
 // linear step of the scheme treats the two members of a pair with the same operation and
 // coefficients of equal size (opposite signs where e enters), so the kernel keeps a pair in one
@@ -60,6 +59,8 @@
 #include "dugks_step3d.cuh"
 
 namespace dugks {
+
+namespace ws27 {  // the D3Q19 kernel (dugks_step3d_ws.cuh) has parts of the same names
 
 // Opposite pairs and the per-cell layout of the ring.
 template <int Q>
@@ -101,7 +102,7 @@ struct Pr {
         return nnz(NP) == 0 && CS % 4 == 2;
     }
 };
-static_assert(Pr<19>::layout_ok() && Pr<27>::layout_ok(), "velocity order without opposite pairs at k, Q - 1 - k");
+static_assert(Pr<27>::layout_ok(), "velocity order without opposite pairs at k, Q - 1 - k");
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
@@ -126,20 +127,16 @@ struct ShapeWS {
     static constexpr int TXI = RX - 2, TYI = RY - 2;  // inner columns
     static constexpr int CS = P::CS;                  // ring floats per cell
     // numbers per interface: the polynomial's, or (with a force) the brackets of the crossing pairs
-    static constexpr int NV = FORCE ? 2 * P::NX : (Q == 27 ? 10 : 8);
-    static constexpr bool U0 = Q == 19;               // u0 passes through shared memory (D3Q27: no room)
-    static constexpr int UP = 2 * P::NP;              // u0 pairs of one column and plane
-    static constexpr int NSLOT = 4, NU0 = U0 ? 3 : 0;
-    static constexpr int NUC = TYI * RX;              // columns that update (rows 1 .. TYI)
+    static constexpr int NV = FORCE ? 2 * P::NX : 10;
+    static constexpr int NSLOT = 4;
     static constexpr int PLANE = RY * RX * CS;
     // Without a force every row forms the numbers of both its y interfaces from the parts A_y, B_y of
     // its neighbours (double-buffered, one barrier per plane); with one, where they are many, each
     // interface's are formed once and published behind a second barrier.
     static constexpr bool BOTH_Y = !FORCE;
-    // ring; A_y and B_y of all rows; numbers at +y of rows 0..RY-2; wall terms of the low and high y
-    // wall; u0 pairs and rest of rows 1..TYI
+    // ring; A_y and B_y of all rows; numbers at +y of rows 0..RY-2; wall terms of the low and high y wall
     static constexpr int XB = (BOTH_Y ? 2 : 1) * RY * RX * 8, YV = BOTH_Y ? 0 : (RY - 1) * RX * NV, WT = 2 * 2 * RX * 2 * P::NX;
-    static constexpr size_t FLOATS = (size_t)NSLOT * PLANE + XB + YV + WT + (size_t)NU0 * NUC * (UP + 1);
+    static constexpr size_t FLOATS = (size_t)NSLOT * PLANE + XB + YV + WT;
     static_assert(PLANE % 4 == 0 && XB % 4 == 0 && YV % 4 == 0 && WT % 4 == 0, "vector accesses must stay aligned");
     static constexpr int BX = 32 + (sizeof(S) == 4 ? 4 : 8);  // TMA box width (start rounded down)
     static constexpr size_t STAGE_BYTES = (size_t)Q * RY * BX * sizeof(S);
@@ -166,14 +163,14 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 
 // Step 1 (eq. (24) with eq. (6)) for one cell on pairs: G[j] = (g~_j, g~_{Q-1-j}), g9 the rest
 // velocity, Gh the acceleration / c at t_n (FORCE). Writes the cell's ring entry o (fbar+ and its
-// moments) and, with `u` non-null, u0 = g~ + 4/3 (fbar+ - g~) (pairs to u, the rest velocity to *ur).
+// moments).
 // The momentum sums are exact as in moments<Q, float, true>: heads on the grid of the cell's largest
 // |g| are summed without rounding (pair by pair: the head sums of the first and second members,
 // then their difference), tails separately, one rounding at the end. The equilibrium pair is
 // geq_pair's, the relaxation relax's, one packed operation per pair.
 template <int Q, bool FORCE>
-__device__ __forceinline__ void step1_pairs(const float2 *G, float g9, const float Gh[3], const Coef<float> &cf, float *o,
-                                            float *u, float *ur) {
+__device__ __forceinline__ void step1_pairs(const float2 *G, float g9, const float Gh[3], const Coef<float> &cf,
+                                            float *o) {
     using P = Pr<Q>;
     float2 Rs = G[0];
 #pragma unroll
@@ -207,14 +204,13 @@ __device__ __forceinline__ void step1_pairs(const float2 *G, float g9, const flo
     if (FORCE) gm = dotD<3, float>(Gh, m) * cf.inv_rho0;
     const float base = fmaf(-1.5f * cf.inv_rho0, mm, drho);
     const float c45 = 4.5f * cf.inv_rho0;
-    const float2 B2 = f2(cf.b1, cf.b1), T43 = f2(4.0f / 3.0f, 4.0f / 3.0f);
+    const float2 B2 = f2(cf.b1, cf.b1);
     float f9;
     {
         const float geq = wmul<Q, float>(P::NP, base);
         float inc = cf.b1 * (geq - g9);
         if (FORCE) inc = fmaf(cf.c1, 3.0f * (0.0f - gm) * fmaf((float)Lat<Q>::template wt<double>(P::NP), cf.rho0, geq), inc);
         f9 = g9 + inc;
-        if (u) *ur = fmaf(4.0f / 3.0f, inc, g9);
     }
     // moments of fbar+: Ps[a] sums the pairs whose first member has e_a = +1, Ns[a] those with -1
     // (the second member then counts the other way)
@@ -243,10 +239,8 @@ __device__ __forceinline__ void step1_pairs(const float2 *G, float g9, const flo
             const float c3 = 3.0f * cf.c1;
             const float2 I = __ffma2_rn(f2(c3 * (ge - gm), c3 * (-ge - gm)), FEQ, __fmul2_rn(B2, D));
             F = __fadd2_rn(G[j], I);
-            if (u) st2(u + 2 * j, __ffma2_rn(T43, I, G[j]));
         } else {
             F = __ffma2_rn(B2, D, G[j]);
-            if (u) st2(u + 2 * j, __ffma2_rn(__fmul2_rn(T43, B2), D, G[j]));
         }
         st2(o + 2 * j, F);
         if constexpr (ex > 0) Ps[0] = __fadd2_rn(Ps[0], F);
@@ -333,8 +327,8 @@ __device__ __forceinline__ void face_G3(const StepParams &p, int d, int x, int y
 // A y or z wall interface by the direct path (all velocities reconstructed, steps 3-7): the
 // interface normal to d between the cell (row, lane) at plane pl and the next cell along d, gfd its
 // index along d. T: f - (1 - b7) F of the crossing pairs, divided by 1 - b7, so that e_d T added to
-// the regular La of the cell below (subtracted above) makes the wall's f its flux. Out of line:
-// one row of a wall tile, and the first and last plane, take it.
+// the regular La of the cell below (subtracted above) makes the wall's f its flux. One row of
+// a wall tile, and the first and last plane, take it.
 template <int Q, bool FORCE, int d>
 __device__ __forceinline__ void wall_term(const StepParams &p, const WsCtx &c, int row, int pl, int gfd, float2 *T) {
     using P = Pr<Q>;
@@ -467,8 +461,6 @@ __global__ void __launch_bounds__(512, 1)
     float *xb = ring + K::NSLOT * K::PLANE;            // [2][RY][32][8]: A_y, B_y (by the plane's parity)
     float *yv = xb + K::XB;                            // [rows 0..RY-2][NV][32]: numbers at +y
     float *wt = yv + K::YV;                            // [2][2][32][2 NX]: terms of the low / high y wall
-    float *u0b = wt + K::WT;                           // [NU0][rows 1..TYI][32][UP]
-    float *u0r = u0b + K::NU0 * K::NUC * K::UP;        // [NU0][rows 1..TYI][32]: rest velocity
     unsigned char *stage = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw + K::STAGE_OFF) + 127) & ~(uintptr_t)127);
     uint64_t *full = reinterpret_cast<uint64_t *>(stage + K::BAR_OFF);
@@ -493,8 +485,7 @@ __global__ void __launch_bounds__(512, 1)
     const bool perx = p.bc[0] == 0, pery = p.bc[2] == 0, perz = p.bc[4] == 0;
     const S *src = reinterpret_cast<const S *>(p.src);
     S *dst = reinterpret_cast<S *>(p.dst);
-    // planes z0 - 1 .. z1 in order: n = pz - (z0 - 1) selects ring slot n % 4 (phase n / 4) and u0
-    // slot n % 3
+    // planes z0 - 1 .. z1 in order: n = pz - (z0 - 1) selects ring slot n % 4 (phase n / 4)
     auto nidx = [&](int pz) __attribute__((always_inline)) { return pz - (z0 - 1); };
     auto slot_of = [&](int pz) __attribute__((always_inline)) { return nidx(pz) & 3; };
     auto R = [&](int slot, int r, int l) __attribute__((always_inline)) -> float * {
@@ -532,9 +523,8 @@ __global__ void __launch_bounds__(512, 1)
         const bool yreal = (gy >= 0 && gy < ny) || (pery && gy >= -1 && gy <= ny);
         const bool xghost = !perx && (gx == -1 || gx == nx) && yreal;
         const bool yghost = !pery && (gy == -1 || gy == ny) && gx >= -1 && gx <= nx;
-        const bool urow = K::U0 && row >= 1 && row <= K::TYI;  // columns whose u0 the consumers read
         int m = 0;  // real planes read from the stage so far
-        // step 1 for real plane pz into its ring and u0 slots; false: a wait gave up (every
+        // step 1 for real plane pz into its ring slot; false: a wait gave up (every
         // producer thread learns it at the same barrier)
         auto make_plane = [&](int pz) __attribute__((always_inline)) -> bool {
             const int gz = wrap_idx(pz, nz);
@@ -578,8 +568,7 @@ __global__ void __launch_bounds__(512, 1)
                 const int64_t ci = (int64_t)cx + (int64_t)nx * ((int64_t)cy + (int64_t)ny * gz);
                 cell_G<3, float>(p, ci, ncell, cf.ct, Gh);
             }
-            const int us = (nidx(pz) % 3) * K::NUC + (row - 1) * 32 + lane;
-            step1_pairs<Q, FORCE>(G, g9, Gh, cf, o, urow ? u0b + us * K::UP : nullptr, u0r + us);
+            step1_pairs<Q, FORCE>(G, g9, Gh, cf, o);
             return true;
         };
         // step 2 (reading R3: ghost = 2 f0 - f1, x then y): fbar+ and, by linearity, its moments
@@ -739,10 +728,8 @@ __global__ void __launch_bounds__(512, 1)
             V[5] = s2 * m[t];            // S_t
             V[6] = fmaf(wu2, m[u], Pn);  // R_u
             V[7] = s2 * m[u];            // S_u
-            if constexpr (Q == 27) {
-                V[8] = fmaf(wu2, m[u], V[4]);   // base + 4.5 (m_x^2 + m_y^2 + m_z^2) / rho0
-                V[9] = 2.0f * wt2 * m[u];       // 9 m_t m_u / rho0
-            }
+            V[8] = fmaf(wu2, m[u], V[4]);   // base + 4.5 (m_x^2 + m_y^2 + m_z^2) / rho0
+            V[9] = 2.0f * wt2 * m[u];       // 9 m_t m_u / rho0
         } else {
             // Y = b7 X + t (rho0 + X), X = q +- 3 e.m, t = 3 c7 (+-G.e - G.m / rho0)
             const float c73 = 3.0f * cf.c7, gm = c73 * (dotD<3, float>(Gh, m) * cf.inv_rho0);
@@ -1041,22 +1028,16 @@ __global__ void __launch_bounds__(512, 1)
                 });
             }
             const float mk = -cf.two_kappa, b7 = cf.b7;
-            const int us = (nidx(kz) % 3) * K::NUC + (row - 1) * 32 + lane;
-            const float *u0 = u0b + us * K::UP;
             const int64_t off = (int64_t)kz * p.plane + (int64_t)gy * p.px + gx;
             const CellRandom rnd(seed, off);
             sfor<NP>([&](auto jc) {
                 constexpr int j = jc, ex = P::e(j, 0), ey = P::e(j, 1), ez = P::e(j, 2), nn = P::nnz(j);
                 constexpr int i = ez != 0 ? P::pos(2, j) : 0;
                 const float2 f = ld2(cur + 2 * j);
-                float2 u;
-                if constexpr (K::U0) {
-                    u = ld2(u0 + 2 * j);
-                } else {  // eq. (25): 4/3 fbar+ - 1/3 g~
-                    const float2 g = f2((float)Store<S>::ld(src + j * p.dstride + off),
-                                        (float)Store<S>::ld(src + (Q - 1 - j) * p.dstride + off));
-                    u = __ffma2_rn(f2(1.0f / 3.0f, 1.0f / 3.0f), sub2(f, g), f);
-                }
+                // eq. (25): 4/3 fbar+ - 1/3 g~
+                const float2 g = f2((float)Store<S>::ld(src + j * p.dstride + off),
+                                    (float)Store<S>::ld(src + (Q - 1 - j) * p.dstride + off));
+                const float2 u = __ffma2_rn(f2(1.0f / 3.0f, 1.0f / 3.0f), sub2(f, g), f);
                 // La: the part of plane kz + 1; then the next plane's, with the part of this one
                 float2 l = La[j], ln, dx, dy;
                 planar(jc, nxt, ln, dx, dy);
@@ -1127,13 +1108,7 @@ __global__ void __launch_bounds__(512, 1)
                 store_state<S>(dst + j * p.dstride + off, v.x, sizeof(S) == 2 ? rnd.template bits<j>() : 0u);
                 store_state<S>(dst + (Q - 1 - j) * p.dstride + off, v.y, sizeof(S) == 2 ? rnd.template bits<Q - 1 - j>() : 0u);
             });
-            float ur;
-            if constexpr (K::U0) {
-                ur = u0r[us];
-            } else {
-                const float f = cur[P::REST];
-                ur = fmaf(1.0f / 3.0f, f - (float)Store<S>::ld(src + NP * p.dstride + off), f);
-            }
+            const float f0 = cur[P::REST], ur = fmaf(1.0f / 3.0f, f0 - (float)Store<S>::ld(src + NP * p.dstride + off), f0);
             store_state<S>(dst + NP * p.dstride + off, ur, sizeof(S) == 2 ? rnd.template bits<NP>() : 0u);
         }
 #pragma unroll
@@ -1145,22 +1120,6 @@ __global__ void __launch_bounds__(512, 1)
         // this thread has read the ring slot of plane kz - 1 for the last time
         release(kz - 1);
     }
-}
-
-// z chunks per tile column for one CTA per SM: maximise (useful waves / launched waves) /
-// (1 + 2 / chunk length) (each chunk makes two extra planes of fbar+ in its prologue).
-inline int zchunk_for(int64_t tiles, int nz, int64_t slots) {
-    int best = 1;
-    double best_eff = -1.0;
-    for (int nc = 1; nc <= 16; nc++) {
-        const int zc = (nz + nc - 1) / nc;
-        if (nc > 1 && zc < 8) break;
-        const int ncr = (nz + zc - 1) / zc;
-        const double waves = (double)(tiles * ncr) / (double)slots;
-        const double eff = waves / ceil(waves) / (1.0 + 2.0 / zc);
-        if (eff > best_eff + 1e-9) { best_eff = eff; best = nc; }
-    }
-    return (nz + best - 1) / best;
 }
 
 // One step by the kernel above: 8 producer + 8 consumer warps, one CTA per SM, 32 x 8 columns per tile.
@@ -1193,5 +1152,7 @@ cudaError_t launch_ws(const StepParams &p, cudaStream_t stream) {
     fused_step3d_ws<Q, S, FORCE><<<dim3(tiles_x, tiles_y, nchunks), K::NTHREADS, K::smem_bytes, stream>>>(p, map, zchunk);
     return cudaGetLastError();
 }
+
+}  // namespace ws27
 
 }  // namespace dugks

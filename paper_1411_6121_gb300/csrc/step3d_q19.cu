@@ -76,20 +76,7 @@ static cudaError_t launch_ry(const StepParams &p, cudaStream_t stream) {
     const int tiles_x = (p.nx + K::TXI - 1) / K::TXI;
     const int tiles_y = (p.ny + K::TYI - 1) / K::TYI;
     const int64_t tiles = (int64_t)tiles_x * tiles_y;
-    // number of z chunks: maximise (useful waves / launched waves) / (1 + 2 / chunk length)
-    // (each chunk recomputes two extra planes of fbar+ in its prologue)
-    const int64_t slots = (int64_t)sms * blocks_per_sm;
-    int best = 1;
-    double best_eff = -1.0;
-    for (int nc = 1; nc <= 16; nc++) {
-        const int zc = (p.nz + nc - 1) / nc;
-        if (nc > 1 && zc < 8) break;
-        const int ncr = (p.nz + zc - 1) / zc;
-        const double waves = (double)(tiles * ncr) / (double)slots;
-        const double eff = waves / ceil(waves) / (1.0 + 2.0 / zc);
-        if (eff > best_eff + 1e-9) { best_eff = eff; best = nc; }
-    }
-    const int zchunk = (p.nz + best - 1) / best;
+    const int zchunk = zchunk_for(tiles, p.nz, (int64_t)sms * blocks_per_sm);
     const int nchunks = (p.nz + zchunk - 1) / zchunk;
     dim3 grid(tiles_x, tiles_y, nchunks);
     dim3 block(32, RY);
@@ -102,22 +89,6 @@ static cudaError_t launch_ry(const StepParams &p, cudaStream_t stream) {
     }
     fused_step3d<19, S, RY, FORCE><<<grid, block, K::smem_bytes, stream>>>(p, map, zchunk);
     return cudaGetLastError();
-}
-
-// z chunks per tile column for one CTA per SM: maximise (useful waves / launched waves) /
-// (1 + 2 / chunk length) (each chunk makes two extra planes of fbar+ in its prologue).
-static int zchunk_for(int64_t tiles, int nz, int64_t slots) {
-    int best = 1;
-    double best_eff = -1.0;
-    for (int nc = 1; nc <= 16; nc++) {
-        const int zc = (nz + nc - 1) / nc;
-        if (nc > 1 && zc < 8) break;
-        const int ncr = (nz + zc - 1) / zc;
-        const double waves = (double)(tiles * ncr) / (double)slots;
-        const double eff = waves / ceil(waves) / (1.0 + 2.0 / zc);
-        if (eff > best_eff + 1e-9) { best_eff = eff; best = nc; }
-    }
-    return (nz + best - 1) / best;
 }
 
 // The warp-specialised kernel (dugks_step3d_ws.cuh): 8 producer + 8 consumer warps, one CTA

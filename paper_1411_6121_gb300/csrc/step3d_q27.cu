@@ -28,19 +28,7 @@ static cudaError_t launch27(const StepParams &p, cudaStream_t stream) {
     const int tiles_x = (p.nx + K::TXI - 1) / K::TXI;
     const int tiles_y = (p.ny + K::TYI - 1) / K::TYI;
     const int64_t tiles = (int64_t)tiles_x * tiles_y;
-    // z chunks: maximise (useful waves / launched waves) / (1 + 2 / chunk length), one CTA
-    // per SM (each chunk recomputes two extra planes of fbar+ in its prologue)
-    int best = 1;
-    double best_eff = -1.0;
-    for (int nc = 1; nc <= 16; nc++) {
-        const int zc = (p.nz + nc - 1) / nc;
-        if (nc > 1 && zc < 8) break;
-        const int ncr = (p.nz + zc - 1) / zc;
-        const double waves = (double)(tiles * ncr) / (double)sms;
-        const double eff = waves / ceil(waves) / (1.0 + 2.0 / zc);
-        if (eff > best_eff + 1e-9) { best_eff = eff; best = nc; }
-    }
-    const int zchunk = (p.nz + best - 1) / best;
+    const int zchunk = zchunk_for(tiles, p.nz, sms);  // one CTA per SM
     const int nchunks = (p.nz + zchunk - 1) / zchunk;
     static_assert(!K::TMA, "D3Q27 loads its planes directly");
     CUtensorMap unused;
@@ -64,7 +52,7 @@ int tma_wait_failures_q27() {
 template <class S>
 static cudaError_t launch_s(const StepParams &p, int ry, cudaStream_t stream) {
     const bool force = p.field != nullptr || p.g[0] != 0.0 || p.g[1] != 0.0 || p.g[2] != 0.0;
-    if (ry == 0) return force ? launch_ws<27, S, true>(p, stream) : launch_ws<27, S, false>(p, stream);
+    if (ry == 0) return force ? ws27::launch_ws<27, S, true>(p, stream) : ws27::launch_ws<27, S, false>(p, stream);
     return force ? launch27<S, true>(p, stream) : launch27<S, false>(p, stream);
 }
 
