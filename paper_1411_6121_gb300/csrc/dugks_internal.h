@@ -11,9 +11,16 @@ namespace dugks {
 // Launches a kernel whose blocks may be set up while the work ahead of it in the stream still runs
 // (programmatic stream serialization): the kernel begins with chain_wait(), so it orders after
 // that work all the same, and the gap between two steps of a sequence loses the launch itself
-// (0.4 of 3.8 us per step of an 8 x 32 channel, 0.5 of 30.4 of a 1024^2 cavity).
+// (0.4 of 3.8 us per step of an 8 x 32 channel, 0.5 of 30.4 of a 1024^2 cavity). resident: blocks per SM,
+// sms: SMs. Where the blocks of two steps do not fit the GPU together but an SM holds more than a step gives
+// it, the waiting blocks would fill the SMs unevenly (two blocks here, three there, and the step takes as long
+// as three): there the launch is an ordinary one (2D meshes of 1.5 to 2 blocks per SM where three fit: 5 to
+// 17% a step; everywhere else chaining gains 1 to 12%).
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int resident,
+                           int sms, A... args) {
+    const int64_t blocks = (int64_t)grid.x * grid.y * grid.z;
+    const bool uneven = 2 * blocks > (int64_t)resident * sms && blocks <= (int64_t)(resident - 1) * sms;
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
     c.blockDim = block;
@@ -23,7 +30,7 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     c.attrs = &at;
-    c.numAttrs = 1;
+    c.numAttrs = uneven ? 0 : 1;
     return cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 
@@ -40,7 +47,7 @@ cudaError_t launch_step3d_q27(const StepParams &p, int store, int ry, cudaStream
 // Throughput kernel for D2Q9 with F32/BF16/F16 storage (dugks_step2d.cuh; BF16:
 // dugks_step2d_cell.cuh): ry = block rows, tiles of step2d_tile_columns(store) columns x (ry - 2) rows (ry 0: chosen by the mesh; the results do not
 // depend on it). The batch form walks a work list of (instance, x0, y0) tile origins over
-// params[2 i + parity] on a persistent grid; force: 0 no instance has an acceleration, 1 all have,
+// params[2 i + parity], a block per item (BF16: persistent blocks); force: 0 no instance has an acceleration, 1 all have,
 // 2 some.
 int step2d_tile_columns(int store);
 cudaError_t launch_step2d_q9(const StepParams &p, int store, int ry, cudaStream_t stream);

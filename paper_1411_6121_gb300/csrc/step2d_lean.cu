@@ -28,7 +28,7 @@ int block_rows(int64_t nx, int64_t ny, int sms) {
 template <class S, bool NU, bool FORCE>
 cudaError_t launch(const StepParams &p, cudaStream_t stream) {
     using T = typename Arith<S>::T;
-    static int configured_dev = -1, sms = 1;
+    static int configured_dev = -1, sms = 1, blocks[lean::MAX_RY + 1];
     int dev = 0;
     cudaGetDevice(&dev);
     if (configured_dev != dev) {
@@ -37,13 +37,18 @@ cudaError_t launch(const StepParams &p, cudaStream_t stream) {
                                              (int)lean::smem_bytes<T, FORCE>(lean::MAX_RY));
         if (e != cudaSuccess) return e;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        for (int ry = 3; ry <= lean::MAX_RY; ry++) {
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks[ry], lean::fused_step2d_lean<S, NU, FORCE>, 32 * ry,
+                                                          lean::smem_bytes<T, FORCE>(ry));
+            blocks[ry] = blocks[ry] < 1 ? 1 : blocks[ry];
+        }
         configured_dev = dev;
     }
     const int ry = block_rows(p.nx, p.ny, sms);
     // all tiles along x: a grid's y extent (65,535) would end at 393,210 rows of cells
     const dim3 grid((unsigned)((int64_t)((p.nx + lean::TXI - 1) / lean::TXI) * ((p.ny + ry - 3) / (ry - 2))));
     return launch_chained(lean::fused_step2d_lean<S, NU, FORCE>, grid, dim3(32, ry), lean::smem_bytes<T, FORCE>(ry), stream,
-                          p);
+                          blocks[ry], sms, p);
 }
 
 template <class S, bool NU>

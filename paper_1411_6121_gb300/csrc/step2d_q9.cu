@@ -69,7 +69,8 @@ cudaError_t launch_one(const StepParams &p, int ry, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     if (ry == 0) ry = block_rows(p.nx, p.ny, *r);
     const dim3 grid((p.nx + m2::TXI - 1) / m2::TXI, (p.ny + ry - 3) / (ry - 2));
-    return launch_chained(fused_step2d<S, FORCE>, grid, dim3(32, ry), m2::smem_bytes<FORCE>(ry), stream, p);
+    return launch_chained(fused_step2d<S, FORCE>, grid, dim3(32, ry), m2::smem_bytes<FORCE>(ry), stream, r->blocks[ry],
+                          r->sms, p);
 }
 
 template <class S, int FORCE>
@@ -80,7 +81,7 @@ cudaError_t launch_many(const StepParams *params, const int4 *items, int nitems,
     if (e != cudaSuccess) return e;
     if (nitems < 1) return cudaSuccess;
     return launch_chained(fused_step2d_batch<S, FORCE>, dim3(nitems), dim3(32, ry), m2::smem_bytes<FORCE != 0>(ry), stream,
-                          params, items, parity);
+                          r->blocks[ry], r->sms, params, items, parity);
 }
 
 template <class S>

@@ -14,39 +14,41 @@ using S = __nv_bfloat16;
 template <int RY, bool FORCE>
 cudaError_t launch_one(const StepParams &p, cudaStream_t stream) {
     using K = Shape2<RY, S>;
-    static int configured_dev = -1;
+    static int configured_dev = -1, bps = 1, sms = 1;
     int dev = 0;
     cudaGetDevice(&dev);
     if (configured_dev != dev) {
         cudaError_t e = cudaFuncSetAttribute(fused_step2d_cell<S, RY, FORCE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)K::smem_bytes);
         if (e != cudaSuccess) return e;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fused_step2d_cell<S, RY, FORCE>, 32 * RY, K::smem_bytes);
+        bps = std::max(1, bps);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         configured_dev = dev;
     }
     const dim3 grid((p.nx + K::TXI - 1) / K::TXI, (p.ny + K::TYI - 1) / K::TYI);
-    return launch_chained(fused_step2d_cell<S, RY, FORCE>, grid, dim3(32, RY), K::smem_bytes, stream, p);
+    return launch_chained(fused_step2d_cell<S, RY, FORCE>, grid, dim3(32, RY), K::smem_bytes, stream, bps, sms, p);
 }
 
 template <int RY, bool FORCE>
 cudaError_t launch_many(const StepParams *params, const int4 *items, int nitems, int parity, cudaStream_t stream) {
     using K = Shape2<RY, S>;
-    static int configured_dev = -1, resident = 1;
+    static int configured_dev = -1, bps = 1, sms = 1;
     int dev = 0;
     cudaGetDevice(&dev);
     if (configured_dev != dev) {
         cudaError_t e = cudaFuncSetAttribute(fused_step2d_cell_batch<S, RY, FORCE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::smem_bytes);
         if (e != cudaSuccess) return e;
-        int bps = 1, sms = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fused_step2d_cell_batch<S, RY, FORCE>, 32 * RY, K::smem_bytes);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        resident = std::max(1, bps) * sms;
+        bps = std::max(1, bps);
         configured_dev = dev;
     }
-    const int grid = std::min(nitems, resident);  // persistent: the resident blocks, at most the items
+    const int grid = std::min(nitems, bps * sms);  // persistent: the resident blocks, at most the items
     if (grid < 1) return cudaSuccess;
-    return launch_chained(fused_step2d_cell_batch<S, RY, FORCE>, dim3(grid), dim3(32, RY), K::smem_bytes, stream, params,
-                          items, nitems, parity);
+    return launch_chained(fused_step2d_cell_batch<S, RY, FORCE>, dim3(grid), dim3(32, RY), K::smem_bytes, stream, bps, sms,
+                          params, items, nitems, parity);
 }
 
 template <bool FORCE>
