@@ -53,7 +53,11 @@ int step2d_tile_columns(int store);
 cudaError_t launch_step2d_q9(const StepParams &p, int store, int ry, cudaStream_t stream);
 cudaError_t launch_step2d_batch(const StepParams *params, const int4 *items, int nitems, int parity, int store,
                                 int ry, int force, cudaStream_t stream);
-cudaError_t launch_step2d_q9_bf16(const StepParams &p, int ry, cudaStream_t stream);
+// One cell per thread (dugks_step2d_cell.cuh): BF16 with 4, 8 or 16 rows, F32 and F16 with 8.
+// step2d_cell_warps: the warps that a step of that kernel (F32, F16) gives the busiest SM, 0 if its blocks are
+// not all resident at once.
+cudaError_t launch_step2d_cell(const StepParams &p, int store, int ry, cudaStream_t stream);
+int step2d_cell_warps(const StepParams &p, int store, bool force);
 cudaError_t launch_step2d_batch_bf16(const StepParams *params, const int4 *items, int nitems, int parity, int ry,
                                      bool force, cudaStream_t stream);
 

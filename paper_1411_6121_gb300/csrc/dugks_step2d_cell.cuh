@@ -1,6 +1,7 @@
-// dugks_step2d_cell.cuh -- the D2Q9 throughput kernel with one cell per thread, for BF16 storage.
+// dugks_step2d_cell.cuh -- the D2Q9 throughput kernel with one cell per thread: BF16 storage, and the F32
+// and F16 meshes whose step is the latency of a block (the rule stands in step2d_q9.cu).
 //
-// F32 and F16 storage run dugks_step2d.cuh, which takes 0.75 of the time of this form. BF16 stays
+// Larger F32 and F16 meshes run dugks_step2d.cuh, which takes 0.75 of the time of this form. BF16 stays
 // here because its rounding noise is part of the result: on the force-driven 8 x 32 channel the
 // time-averaged error against the parabola is 4.8% below FP32's with this kernel's sequence of
 // roundings and 18% above it with the other's (any change of the FP32 arithmetic ahead of the

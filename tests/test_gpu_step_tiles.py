@@ -44,6 +44,15 @@ def test_d2q9_tile_edges(shape, flow):
     assert np.abs(got - ref).max() < 2e-6 * np.abs(ref).max()
 
 
+@pytest.mark.parametrize("flow", sorted(FLOWS))
+@pytest.mark.parametrize("shape", [(9, 724), (31, 604), (78, 883), (1140, 49)])
+def test_d2q9_either_side_of_the_one_cell_rule(shape, flow):
+    """Meshes that the one-cell kernel takes (the first three) and one beyond its rule."""
+    cfg = dict(shape=shape, q=9, nu=0.05, dt=0.5, **FLOWS[flow])
+    ref, got = _pair(cfg, 10)
+    assert np.abs(got - ref).max() < 2e-6 * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("flow", ["box", "channel"])
 def test_d2q9_bits_do_not_depend_on_the_block(flow):
     cfg = dict(shape=(67, 31), q=9, nu=0.05, dt=0.5, **FLOWS[flow])

@@ -14,6 +14,7 @@ pytestmark = pytest.mark.gpu
 
 CASES = {
     "2d_odd": dict(shape=(61, 37), q=9, bcs=W.cavity_bcs(2, 0.1)),
+    "2d_tall": dict(shape=(40, 300), q=9, bcs=W.cavity_bcs(2, 0.1)),
     "2d_forced": dict(shape=(128, 33), q=9, bcs=W.channel_bcs(2), g=(1e-4, -2e-5, 0.0)),
     "d3q27": dict(shape=(35, 13, 9), q=27, bcs=W.cavity_bcs(3, 0.1)),
     "d3q27_forced": dict(shape=(31, 14, 6), q=27, bcs=W.channel_bcs(3), g=(1e-4, -2e-5, 3e-5)),
