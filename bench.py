@@ -318,7 +318,7 @@ def run_e2e(torch, steps, dev, trials=3, handles=2):
 
 def run_batched(torch, steps, warmup, dev):
     """The batched form: 64 force-driven D2Q9 channels of uneven sizes (32x16 to 512x256,
-    Re 10-500, seeded) with per-cell acceleration fields, one persistent launch per step,
+    Re 10-500, seeded) with per-cell acceleration fields, one launch per step,
     CUDA-graph replay, autotuned tile."""
     from paper_1411_6121_gb300 import dugks
     from paper_1411_6121_gb300 import workloads as W
@@ -353,8 +353,8 @@ def run_batched(torch, steps, warmup, dev):
             "cells": cells, "tile": list(tile), "steps": steps,
             "roofline": {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
                          "bytes_per_cell_update": bpc, "peak_source": src,
-                         "note": "events around the graph replay of all steps (one persistent launch each)"},
-            "note": "64 D2Q9 channels, one persistent launch per step replayed as a CUDA graph"}
+                         "note": "events around the graph replay of all steps (one launch each)"},
+            "note": "64 D2Q9 channels, one launch per step replayed as a CUDA graph"}
 
 
 ADJ_STEPS, ADJ_EVERY = 2000, 100

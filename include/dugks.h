@@ -122,9 +122,9 @@ typedef struct {
     void *stream;           /* cudaStream_t to run on (default NULL: own stream)     */
     int32_t use_graph;      /* 1: dugks_step replays a captured CUDA graph (default) */
     int32_t tile_x, tile_y; /* 0: default tile. Throughput kernels (kernel 0, F32/BF16/F16
-                               storage): tile_y = thread-block rows (D2Q9: 4, 8 or 16, by
-                               default chosen by the mesh, with the same results;
-                               D3Q19: 8 or 10, D3Q27: 8 take the non-specialised
+                               storage): tile_y = thread-block rows (D2Q9: 4, 8 or 16, with
+                               the same results; by default the rows, and on small F32
+                               and F16 meshes the kernel, are chosen by the mesh; D3Q19: 8 or 10, D3Q27: 8 take the non-specialised
                                kernel; default the warp-specialised one), tile_x ignored.
                                Reference
                                kernel: tile_x x tile_y = 32x8 or 16x8                   */
@@ -243,8 +243,8 @@ int dugks_adjoint_wall(dugks_t h, double *dL_dwall);
 /* ---- batched form: many independent 2D instances ---------------------------------------
  * A batch advances `count` independent D2Q9 instances (each its own mesh, viscosity,
  * acceleration and boundaries; shared dt, RT, rho0 and storage from opts) together: one time
- * step of the whole batch is one persistent kernel launch over a work list of (instance,
- * tile) items, largest instances first, and dugks_batch_step replays n such launches as one
+ * step of the whole batch is one kernel launch over a work list of (instance, tile) items,
+ * largest instances first, and dugks_batch_step replays n such launches as one
  * captured CUDA graph. The per-instance scheme is exactly that of dugks_step (Appendix
  * steps 1-10 of the paper). meshes/nu/forces/bcs: HOST arrays of `count` records (a force
  * field pointer, if any, is a DEVICE [2][ncell] float array read at every step). opts may
@@ -296,7 +296,7 @@ void dugks_batch_destroy(dugks_batch_t b);
  *   out:    HOST [dim+2] doubles: out[0] = ||u - uprev||/||u|| (+inf when have_prev == 0),
  *           out[1] = sum rho, out[2+a] = sum rho0 u_a.
  *   stream: cudaStream_t (NULL: legacy stream); the call synchronises it before returning.
- * Limit: at most 16,777,216 cells (256^3; 4096 partial-sum blocks of at most 4096 cells);
+ * Limit: at most 16,777,216 cells (256^3);
  * larger meshes return DUGKS_E_INVAL with the limit in dugks_last_error(NULL). The first
  * call on a device looks up the array's device address (cudaGetSymbolAddress, with that
  * device current) and caches it. Every call on a device shares the one array: calls that

@@ -44,11 +44,11 @@ cudaError_t launch_step_q27(const StepParams &p, int store, int tx, int ty, cuda
 // (dugks_step3d_ws.cuh, dugks_step3d_ws27.cuh), else the non-specialised one (dugks_step3d.cuh) with ry CTA rows (D3Q27: 8).
 cudaError_t launch_step3d_q19(const StepParams &p, int store, int ry, cudaStream_t stream);
 cudaError_t launch_step3d_q27(const StepParams &p, int store, int ry, cudaStream_t stream);
-// Throughput kernel for D2Q9 with F32/BF16/F16 storage (dugks_step2d.cuh; BF16:
-// dugks_step2d_cell.cuh): ry = block rows, tiles of step2d_tile_columns(store) columns x (ry - 2) rows (ry 0: chosen by the mesh; the results do not
-// depend on it). The batch form walks a work list of (instance, x0, y0) tile origins over
-// params[2 i + parity], a block per item (BF16: persistent blocks); force: 0 no instance has an acceleration, 1 all have,
-// 2 some.
+// Throughput kernel for D2Q9 with F32/BF16/F16 storage (dugks_step2d.cuh; BF16, and small F32 and F16
+// meshes with ry 0: dugks_step2d_cell.cuh): ry = block rows, tiles of step2d_tile_columns(store) columns x
+// (ry - 2) rows; 0: kernel and rows chosen by the mesh (a kernel's results do not depend on the rows). The
+// batch form walks a work list of (instance, x0, y0) tile origins over params[2 i + parity], a block per item
+// (BF16: persistent blocks); force: 0 no instance has an acceleration, 1 all have, 2 some.
 int step2d_tile_columns(int store);
 cudaError_t launch_step2d_q9(const StepParams &p, int store, int ry, cudaStream_t stream);
 cudaError_t launch_step2d_batch(const StepParams *params, const int4 *items, int nitems, int parity, int store,

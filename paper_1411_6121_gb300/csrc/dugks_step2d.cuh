@@ -1,5 +1,6 @@
 // dugks_step2d.cuh -- throughput kernel of the fused DUGKS time step for the D2Q9 velocity
-// set on sm_103a, FP32 arithmetic, F32 and F16 storage (BF16: dugks_step2d_cell.cuh).
+// set on sm_103a, FP32 arithmetic, F32 and F16 storage (BF16, and meshes whose step is the latency of a
+// block: dugks_step2d_cell.cuh; the rule stands in step2d_q9.cu).
 //
 // Same scheme and readings as the reference kernel in dugks_step.cuh (Appendix steps 1-10
 // of arXiv 1411.6121). What bounds a 2D step is instruction issue, so the work is arranged to
@@ -36,8 +37,8 @@
 //    increment form with split weights of dugks_step3d_ws27.cuh gave 0.92 / 0.91, 0.95 / 0.95, 0.91 / 0.88 for 1% of a
 //    batch's time.
 // Measured (us per step, one instance, before / now; before: one cell per thread, 32 x 8 threads, 30
-// warp instructions per cell, 56% issue): 1024^2 cavity 40.0 / 27.2 (16 instructions per cell, 53%
-// issue, 24 warps per SM), 2048^2 155 / 102, 512 x 256 channel 8.8 / 6.8, 8 x 32 channel 3.45 / 3.2 (the
+// warp instructions per cell, 56% issue): 1024^2 cavity 40.0 / 27.2, 2048^2 155 / 102 (15.4 instructions
+// per cell, 54% issue, 24 warps per SM), 512 x 256 channel 8.8 / 6.8, 8 x 32 channel 3.45 / 3.2 (the
 // latency of one block).
 #pragma once
 

@@ -16,8 +16,8 @@
 //  * The interface moments in moment space, by the same formula from the cells' moments.
 //  * Without a force the equilibrium part of f across a cell is combined from five numbers per
 //    interface (dugks_step2d.cuh); with one, from the brackets of the crossing velocities.
-// Measured (us per step, reference kernel / this one): 128^2 graded cavity F64 62 / 29; of that 77% is
-// the FP64 pipe at work (315,344 warp instructions).
+// Measured (us per step, reference kernel / this one): 128^2 graded cavity F64 62 / 29, the FP64 pipe 79%
+// busy with 315,344 warp instructions (616 operations per cell with the tiles' halos).
 #pragma once
 
 #include "dugks_step.cuh"
