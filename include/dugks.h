@@ -250,7 +250,8 @@ int dugks_adjoint_wall(dugks_t h, double *dL_dwall);
  * field pointer, if any, is a DEVICE [2][ncell] float array read at every step). opts may
  * be NULL; opts->tile_x/tile_y pick the tile: 30x2, 30x6 or 30x14, 2, 6 or 14 inner rows of the
  * throughput kernel (32 x 4, 8 or 16 threads; F32/BF16/F16), or 32x8, 16x8, 32x4 or 64x4 of the reference
- * kernel; default 30x6.
+ * kernel; default 30x6. An instance has the bits of a single handle with the same kernel and rows asked for
+ * (throughput tiles: kernel 0 and tile_y = 4, 8 or 16); a handle left to choose may take another kernel.
  * Errors as for the single-instance calls; dugks_batch_last_error(b) gives the reason
  * (NULL b: the last failed dugks_batch_create in this thread). */
 typedef struct dugks_batch_s *dugks_batch_t;

@@ -202,10 +202,14 @@ int build_items(dugks_batch_t b) {
 // formed. 64 instances of 32 x 16 to 512 x 256 cells, 36 MB, in ms, by the driver alone / now: into fresh arrays
 // 38 / 3.5, into arrays used before 1.9 / 1.6, into page-locked ones 1.6 / 1.4.
 cudaError_t read_back(dugks_batch_t b, float *out, const void *d, size_t bytes) {
-    volatile char *o = reinterpret_cast<char *>(out);
-    const size_t page = (size_t)sysconf(_SC_PAGESIZE);
-    for (size_t at = 0; at < bytes; at += page) o[at] = 0;
-    o[bytes - 1] = 0;
+    cudaPointerAttributes attr;
+    if (cudaPointerGetAttributes(&attr, out) != cudaSuccess) cudaGetLastError();
+    else if (attr.type == cudaMemoryTypeUnregistered) {  // a device pointer is left to the copy to refuse
+        volatile char *o = reinterpret_cast<char *>(out);
+        const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+        for (size_t at = 0; at < bytes; at += page) o[at] = 0;
+        o[bytes - 1] = 0;
+    }
     return cudaMemcpyAsync(out, d, bytes, cudaMemcpyDeviceToHost, b->stream);
 }
 

@@ -46,3 +46,15 @@ def test_page_locked_destination(batch):
         out = torch.zeros((3, nx * ny), dtype=torch.float32).pin_memory()
         b._check(b.lib.dugks_batch_moments(b.h, i, C.c_void_p(out.data_ptr()), 0))
         assert np.array_equal(out.numpy(), want[i])
+
+
+def test_device_pointer_passed_as_host(batch):
+    """The copy refuses it (or makes it, where the driver does): the host never writes through it."""
+    import torch
+    b, want = batch
+    nx, ny = SHAPES[2]
+    out = torch.zeros((3, nx * ny), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    rc = b.lib.dugks_batch_moments(b.h, 2, C.c_void_p(out.data_ptr()), 0)
+    assert rc != 0 or np.array_equal(out.cpu().numpy(), want[2])
+    assert np.array_equal(b.moments(2), want[2])
